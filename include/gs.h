@@ -82,7 +82,8 @@ typedef struct gs_config {
     int32_t fwd_batch;            /* Gaussians staged per round in gs_render_fwd: 0 = default;
                                      tile 8: 64/128/256, tile 16: 64/128/256, tile 32: 128/256 */
     int32_t bwd_batch;            /* the same for the adjoint: 0 = default; tile 8: 64/128/256,
-                                     tile 16: 32/64/128, tile 32: 32 */
+                                     tile 16: 32/64/128 (large launches stage 32 whichever of
+                                     them is asked for), tile 32: 32 */
     int32_t mip_filter;           /* 1: the dilation is a 2-D low-pass filter that keeps the splat's
                                      integral (multi-scale training, Sec. 4.3): opacity times
                                      sqrt(rho), rho = det(Sigma2D) / det(Sigma2D + dilation I)
@@ -245,7 +246,8 @@ int gs_render_fwd(const gs_projected* p, const gs_pairs* pairs, const gs_frame* 
 /* Measurement (not a step of the method): gs_render_fwd with the same
  * arguments and outputs, run by a counting instantiation of its kernel that
  * also writes counts [3] (device, uint64, overwritten): [0] the warp hits its
- * box test passes (each runs the compositing step on 32 lanes), [1] the lane
+ * block test passes, in units of 32 pixels (a hit that runs the compositing
+ * step on 64 pixels counts twice), [1] the
  * evaluations of pixels not yet terminated at those hits, [2] the evaluations
  * that composite (alpha >= alpha_min, before termination) - the (pixel,
  * Gaussian) work the compositing definition requires (Sec. 4.3; the 3DGS

@@ -40,6 +40,13 @@ __device__ __forceinline__ float fast_exp2(float x) {
     return y;
 }
 
+// log2 x on the MUFU unit (PTX lg2.approx), where an absolute error of 1e-6 does no harm.
+__device__ __forceinline__ float fast_log2(float x) {
+    float y;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
 // Hardware reciprocal approximation (MUFU), for x away from 0 and infinity.
 __device__ __forceinline__ float fast_rcp(float x) {
     float y;

@@ -1,5 +1,9 @@
 // Front-to-back alpha compositing (K5) and its adjoint (K6).
 //
+// Two pairs of kernels. 16 x 16 tiles in launches large enough to fill the GPU
+// with them take k_blocks_fwd and k_rows_bwd (further down); the other tile sizes
+// and small launches take k_render_fwd and k_render_bwd, described here:
+//
 // One CTA of TILE x TILE threads per tile (TILE = 8, 16 or 32), one pixel per
 // thread; each warp owns an 8x4 block of pixels so a small splat touches few
 // warps. Each tile's depth-ordered list is walked in batches staged in shared
@@ -454,6 +458,710 @@ __global__ void __launch_bounds__(TILE * TILE) k_render_bwd(gs_frame f, gs_confi
 }
 
 // ---------------------------------------------------------------------------
+// 16 x 16 tiles, large launches. Both kernels are bound by instruction issue, so
+// both put two pixels into the halves of the packed FP32 instructions
+// (fma/mul/add.rn.f32x2: two FP32 operations, each rounded as the scalar one, in
+// one issue slot), give each lane more than one pixel, and drop a Gaussian from a
+// block of pixels that none of its pixels can reach alpha_min in before the block
+// spends anything on it. Images, transmittances and contributor counts are the
+// bits of k_render_fwd; the adjoint keeps that of k_render_bwd but for the
+// roundings of the colour and opacity sums.
+// ---------------------------------------------------------------------------
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ f32x2 both(float v) { return pack2(v, v); }
+__device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+template <bool B>
+struct BoolC {
+    static constexpr bool value = B;
+};
+
+constexpr int kFastTile = 16;
+
+// A list entry as one lane stages it: the exponent coefficients in base 2, e =
+// A dx^2 + B dx dy + C dy^2, the negated centre, opacity, colour, depth, and a
+// bit for each block of the tile in which its alpha can reach alpha_min (bit
+// column + COLS * row).
+//
+// `plain` marks a Gaussian at which the exponent cannot round to a positive
+// value and alpha cannot reach alpha_max, so that a batch of plain ones does
+// without those two tests: with B^2 <= 4 A C (1 - d) the exact exponent is at
+// most -(d/2)(|A| dx^2 + |C| dy^2) while the rounding of its five operations adds
+// at most 8 * 2^-24 (|A| dx^2 + |C| dy^2), less than that for d = 1e-5; then
+// 2^e <= 1 + 2^-22 and o 2^e < alpha_max for o < alpha_max (1 - 1e-6).
+struct Entry {
+    float nx, ny, A, B, C, o, r, g, b, z;
+    unsigned blocks;
+    bool plain;
+};
+
+// COLS x ROWS blocks of 16 / COLS by 16 / ROWS pixels from the tile's first pixel
+// centre (tx0, ty0). A block is kept when the exponent's maximum over the
+// rectangle of its pixel centres - on the two edges that face the Gaussian's
+// centre, or 0 inside - reaches log2(alpha_min / o), with 0.2% + 0.02 to spare.
+// That holds for ellipses that are not too thin (d = 1e-3 in the bound above
+// keeps the rounding of the exponent below 1e-3 of it); the others take the
+// bounding box of stage(). Against the box alone this drops a fifth of the 8x4
+// blocks and a sixth of the 8x8 blocks of the synthetic 1080p scenes.
+template <int COLS, int ROWS>
+__device__ __forceinline__ Entry load_entry(const float2* __restrict__ mean2d, const float4* __restrict__ conic_opa,
+                                            const float4* __restrict__ rgb_depth, uint32_t idx, float tx0, float ty0,
+                                            float alpha_min, float alpha_max) {
+    constexpr float BW = 16 / COLS, BH = 16 / ROWS;
+    const float2 xy = mean2d[idx];
+    const float4 co = conic_opa[idx], rgb = rgb_depth[idx];
+    Entry e;
+    e.nx = -xy.x; e.ny = -xy.y;
+    e.A = -0.5f * kLog2e * co.x; e.B = -kLog2e * co.y; e.C = -0.5f * kLog2e * co.z; e.o = co.w;
+    e.r = rgb.x; e.g = rgb.y; e.b = rgb.z; e.z = rgb.w;
+    const bool conic = e.A < 0.f && e.C < 0.f && e.A > -1e15f && e.C > -1e15f;
+    const float ac4 = 4.f * (e.A * e.C), bb = e.B * e.B;
+    e.plain = conic && bb <= (1.f - 1e-5f) * ac4 && e.o < alpha_max * (1.f - 1e-6f);
+    unsigned m = 0;
+    if (!(e.o >= alpha_min)) {
+        // can never reach alpha_min
+    } else if (conic && bb <= (1.f - 1e-3f) * ac4) {
+        const float low = 1.002f * (fast_log2(alpha_min) - fast_log2(e.o)) - 0.02f;
+        const float sx = -0.5f * e.B * fast_rcp(e.A);  // along a row dy the maximum is at sx dy
+        const float sy = -0.5f * e.B * fast_rcp(e.C);  // along a column dx at sy dx
+#pragma unroll
+        for (int c = 0; c < COLS; c++) {
+            const float X0 = (tx0 + BW * c) + e.nx, X1 = (tx0 + (BW * c + (BW - 1.f))) + e.nx;
+            const float ex = fminf(fmaxf(0.f, X0), X1);  // the column of centres nearest to the Gaussian's
+            const float vs = sy * ex, be = e.B * ex, ae = e.A * ex * ex;
+#pragma unroll
+            for (int r = 0; r < ROWS; r++) {
+                const float Y0 = (ty0 + BH * r) + e.ny, Y1 = (ty0 + (BH * r + (BH - 1.f))) + e.ny;
+                const float ey = fminf(fmaxf(0.f, Y0), Y1);
+                const float vy = fminf(fmaxf(vs, Y0), Y1);       // the maximum on column ex
+                const float ux = fminf(fmaxf(sx * ey, X0), X1);  // and on row ey
+                const float e1 = ae + vy * (be + e.C * vy);
+                const float e2 = e.C * ey * ey + ux * (e.B * ey + e.A * ux);
+                if (!(fmaxf(e1, e2) < low)) m |= 1u << (c + COLS * r);
+            }
+        }
+    } else {
+        float2 xy2;
+        float4 abco, c2, box;
+        stage(mean2d, conic_opa, rgb_depth, idx, alpha_min, xy2, abco, c2, box);
+#pragma unroll
+        for (int c = 0; c < COLS; c++)
+#pragma unroll
+            for (int r = 0; r < ROWS; r++)
+                if (box.x <= tx0 + (BW * c + (BW - 1.f)) && box.z >= tx0 + BW * c &&
+                    box.y <= ty0 + (BH * r + (BH - 1.f)) && box.w >= ty0 + BH * r)
+                    m |= 1u << (c + COLS * r);
+    }
+    e.blocks = m;
+    return e;
+}
+
+// ---------------------------------------------------------------------------
+// Forward: four warps per tile, each warp an 8x8 block, each lane two pixels four
+// rows apart. FB list entries are staged per round by the whole CTA.
+// ---------------------------------------------------------------------------
+struct __align__(16) FwdRow {
+    float nx, ny, A, B;
+    float C, o, r, g;
+    float b, z, unused0, unused1;
+};
+
+// One pixel's forward step by predicated instructions: p = alpha reaches
+// alpha_min (and, with ALL, the exponent is not positive), q = p and the pixel
+// goes on, r = p and it terminates here. T carries a second meaning in its sign:
+// a pixel that has terminated (or lies outside the view) keeps its transmittance
+// with the sign set, so that T (1 - alpha) < t_min holds at every later Gaussian.
+// Predicated FMAs instead of selects: selects and compares share the half-rate
+// ALU pipe.
+struct FwdPixel {
+    float T, cr, cg, cb, cz;
+    int last;  // the batch's last composited Gaussian, or -1
+};
+template <bool ALL>
+__device__ __forceinline__ void composite(FwdPixel& s, float e, float alpha, float aT, float nT, float alpha_min,
+                                          float t_min, float r, float g, float b, int pos) {
+    if (ALL) {
+        asm("{\n\t.reg .pred p, q, r;\n\t"
+            "setp.leu.f32 p, %5, 0f00000000;\n\t"
+            "setp.ge.and.f32 p, %6, %9, p;\n\t"
+            "setp.lt.and.f32 r|q, %8, %10, p;\n\t"
+            "@q fma.rn.f32 %1, %7, %11, %1;\n\t"
+            "@q fma.rn.f32 %2, %7, %12, %2;\n\t"
+            "@q fma.rn.f32 %3, %7, %13, %3;\n\t"
+            "@q sub.rn.f32 %0, %0, %7;\n\t"
+            "@q mov.b32 %4, %14;\n\t"
+            "@r or.b32 %0, %0, 0x80000000;\n\t}"
+            : "+f"(s.T), "+f"(s.cr), "+f"(s.cg), "+f"(s.cb), "+r"(s.last)
+            : "f"(e), "f"(alpha), "f"(aT), "f"(nT), "f"(alpha_min), "f"(t_min), "f"(r), "f"(g), "f"(b), "r"(pos));
+    } else {
+        asm("{\n\t.reg .pred p, q, r;\n\t"
+            "setp.ge.f32 p, %5, %8;\n\t"
+            "setp.lt.and.f32 r|q, %7, %9, p;\n\t"
+            "@q fma.rn.f32 %1, %6, %10, %1;\n\t"
+            "@q fma.rn.f32 %2, %6, %11, %2;\n\t"
+            "@q fma.rn.f32 %3, %6, %12, %3;\n\t"
+            "@q sub.rn.f32 %0, %0, %6;\n\t"
+            "@q mov.b32 %4, %13;\n\t"
+            "@r or.b32 %0, %0, 0x80000000;\n\t}"
+            : "+f"(s.T), "+f"(s.cr), "+f"(s.cg), "+f"(s.cb), "+r"(s.last)
+            : "f"(alpha), "f"(aT), "f"(nT), "f"(alpha_min), "f"(t_min), "f"(r), "f"(g), "f"(b), "r"(pos));
+    }
+}
+
+// 1M Gaussians, eight 1080p views: 1.92 -> 1.21 ms against k_render_fwd<16, 256>
+// (86% of issue slots, FMA and ALU pipes about half busy); with two pixels side by
+// side and the mask scan as before 1.36 ms, the exact block test and its cheaper
+// staging (one log2 and two reciprocals instead of two roots and two divisions)
+// 1.30, two hits per loop round 1.21. Four warps per tile leave small launches
+// with too few warps: at 240 tiles 102 against 82 us, at 960 tiles 132 against
+// 133, at 1840 tiles 67 against 78.
+constexpr int kFwdThreads = 128;
+constexpr int kFwdMinTiles = 1216;
+
+// DEPTH and COUNT as for k_render_fwd; counts[0] counts a warp's hit twice, once
+// for each 32 of its 64 pixels.
+template <int FB, bool DEPTH, bool COUNT = false>
+__global__ void __launch_bounds__(kFwdThreads) k_blocks_fwd(gs_frame f, gs_config cfg,
+                                                            const uint32_t* __restrict__ range,
+                                                            const uint32_t* __restrict__ src,
+                                                            const float2* __restrict__ mean2d,
+                                                            const float4* __restrict__ conic_opa,
+                                                            const float4* __restrict__ rgb_depth,
+                                                            float* __restrict__ color, float* __restrict__ t_final,
+                                                            int32_t* __restrict__ n_contrib,
+                                                            float* __restrict__ depth_out,
+                                                            const uint32_t* __restrict__ order, uint32_t* counter,
+                                                            int n_tiles, unsigned long long* counts) {
+    constexpr int NT = kFwdThreads;
+    unsigned long long n_hit = 0, n_eval = 0, n_comp = 0;
+    __shared__ FwdRow s_g[FB];
+    __shared__ uint8_t s_blocks[FB];  // bits 0-3: the warps whose block it touches; bit 4: needs all tests
+    __shared__ int s_item;
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const float alpha_min = cfg.alpha_min, t_min = cfg.t_min;
+    for (int tile = next_tile(order, counter, n_tiles, true, &s_item); tile >= 0;
+         tile = next_tile(order, counter, n_tiles, false, &s_item)) {
+        const int view = view_of_tile(f, tile);
+        const int local = tile - f.tile_base[view];
+        const int tx = local % f.tiles_x[view], ty = local / f.tiles_x[view];
+        const int x = tx * kFastTile + (w & 1) * 8 + (lane & 7), y = ty * kFastTile + (w >> 1) * 8 + (lane >> 3);
+        const int W = f.width[view], H = f.height[view];
+        const bool in0 = x < W && y < H, in1 = x < W && y + 4 < H;
+        const float px = x + 0.5f;
+        const f32x2 py = pack2(y + 0.5f, y + 4.5f);
+        const float tx0 = tx * kFastTile + 0.5f, ty0 = ty * kFastTile + 0.5f;
+        const uint32_t start = range[2 * tile], end = range[2 * tile + 1];
+        FwdPixel s0 = {in0 ? 1.f : -1.f, 0.f, 0.f, 0.f, 0.f, -1}, s1 = {in1 ? 1.f : -1.f, 0.f, 0.f, 0.f, 0.f, -1};
+        int last0 = 0, last1 = 0;  // list positions after the last composited Gaussian
+        auto done = [&]() { return (__float_as_uint(s0.T) & __float_as_uint(s1.T)) >> 31; };
+        for (uint32_t b0 = start; b0 < end; b0 += FB) {
+            if (__syncthreads_and(done())) break;
+#pragma unroll 1
+            for (int j = threadIdx.x; j < FB; j += NT)
+                if (b0 + j < end) {
+                    const Entry e = load_entry<2, 2>(mean2d, conic_opa, rgb_depth, src[b0 + j], tx0, ty0, alpha_min,
+                                                     cfg.alpha_max);
+                    s_blocks[j] = (uint8_t)(e.blocks | (e.plain ? 0u : 16u));
+                    float4* o = reinterpret_cast<float4*>(&s_g[j]);
+                    o[0] = make_float4(e.nx, e.ny, e.A, e.B);
+                    o[1] = make_float4(e.C, e.o, e.r, e.g);
+                    o[2] = make_float4(e.b, e.z, 0.f, 0.f);
+                }
+            __syncthreads();
+            const int cnt = min((uint32_t)FB, end - b0);
+            s0.last = s1.last = -1;
+            for (int k0 = 0; k0 < cnt; k0 += 32) {
+                if (__all_sync(FULL, done())) break;
+                const unsigned bits = k0 + lane < cnt ? s_blocks[k0 + lane] : 0u;
+                const bool hit = (bits >> w) & 1u;
+                unsigned m = __ballot_sync(FULL, hit);
+                const bool all = (__ballot_sync(FULL, bits & 16u) & m) != 0;
+                auto walk = [&](auto all_c) {
+                    constexpr bool ALL = decltype(all_c)::value;
+                    auto one = [&](int k, const FwdRow& G) {
+                        const float dx = px + G.nx;
+                        const f32x2 dy = add2(py, both(G.ny));
+                        // fma(A dx, dx, fma(C dy, dy, (B dx) dy)): the rounding sequence of exponent2,
+                        // the same forward and backward, so that both take identical decisions
+                        const f32x2 in = fma2(mul2(both(G.C), dy), dy, mul2(both(__fmul_rn(G.B, dx)), dy));
+                        const f32x2 e2 = fma2(both(__fmul_rn(G.A, dx)), both(dx), in);
+                        float e[2], a[2], aT[2], nT[2];
+                        unpack2(e2, e[0], e[1]);
+                        unpack2(mul2(both(G.o), pack2(fast_exp2(e[0]), fast_exp2(e[1]))), a[0], a[1]);
+                        if (ALL) {
+                            a[0] = fminf(cfg.alpha_max, a[0]);
+                            a[1] = fminf(cfg.alpha_max, a[1]);
+                        }
+                        const f32x2 T2 = pack2(s0.T, s1.T);
+                        const f32x2 aT2 = mul2(pack2(a[0], a[1]), T2);  // the blending weights
+                        unpack2(aT2, aT[0], aT[1]);
+                        unpack2(fma2(aT2, both(-1.f), T2), nT[0], nT[1]);  // T (1 - alpha)
+                        if (COUNT) {
+                            n_hit += 2;
+                            n_eval += (s0.T > 0.f) + (s1.T > 0.f);
+                        }
+                        composite<ALL>(s0, e[0], a[0], aT[0], nT[0], alpha_min, t_min, G.r, G.g, G.b, k);
+                        composite<ALL>(s1, e[1], a[1], aT[1], nT[1], alpha_min, t_min, G.r, G.g, G.b, k);
+                        if (COUNT) n_comp += (s0.last == k) + (s1.last == k);
+                        if (DEPTH) {  // composited here exactly when this Gaussian is now the last
+                            if (s0.last == k) s0.cz += aT[0] * G.z;
+                            if (s1.last == k) s1.cz += aT[1] * G.z;
+                        }
+                    };
+                    while (m) {
+                        const int ka = k0 + __ffs(m) - 1;
+                        m &= m - 1;
+                        const bool two = m != 0;
+                        const int kb = two ? k0 + __ffs(m) - 1 : ka;
+                        m &= m - 1;
+                        const FwdRow ga = s_g[ka], gb = s_g[kb];
+                        one(ka, ga);
+                        if (two) one(kb, gb);
+                    }
+                };
+                if (all) walk(BoolC<true>{}); else walk(BoolC<false>{});
+            }
+            if (s0.last >= 0) last0 = (int)(b0 - start) + s0.last + 1;
+            if (s1.last >= 0) last1 = (int)(b0 - start) + s1.last + 1;
+        }
+        const int64_t plane = (int64_t)W * H, pix = f.pix_base[view] + (int64_t)y * W + x;
+        const int64_t cbase = 3 * f.pix_base[view] + (int64_t)y * W + x;
+        auto write = [&](const FwdPixel& s, int last, int64_t down) {
+            const float T = fabsf(s.T);
+            color[cbase + down] = s.cr + T * cfg.bg[0];
+            color[cbase + down + plane] = s.cg + T * cfg.bg[1];
+            color[cbase + down + 2 * plane] = s.cb + T * cfg.bg[2];
+            t_final[pix + down] = T;
+            n_contrib[pix + down] = last;
+            if (DEPTH) depth_out[pix + down] = s.cz;
+        };
+        if (in0) write(s0, last0, 0);
+        if (in1) write(s1, last1, 4 * (int64_t)W);
+        __syncthreads();  // shared buffers are reused by the next tile
+    }
+    if (COUNT) {
+        for (int o = 16; o > 0; o >>= 1) {
+            n_eval += __shfl_xor_sync(FULL, n_eval, o);
+            n_comp += __shfl_xor_sync(FULL, n_comp, o);
+        }
+        if (lane == 0) {
+            atomicAdd(&counts[0], n_hit);  // every lane counted the warp's hits; lane 0 reports them once
+            atomicAdd(&counts[1], n_eval);
+            atomicAdd(&counts[2], n_comp);
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Adjoint: one warp per tile, each quad of lanes owning one 8x4 block of pixels
+// and each lane one row of eight of them. The quads walk lists of their own: at
+// any time the eight quads work on eight different Gaussians, so a block costs
+// nothing for a Gaussian that does not touch it, no barrier joins warps, a
+// Gaussian's sums over a row stay in registers, and what it costs beside its
+// pixels - loads, list and loop, the reduction over rows - is paid once per eight
+// blocks.
+//
+// 1M Gaussians, eight 1080p views: 4.43 -> 2.33 ms against k_render_bwd<16, 64>
+// (115 instead of 248 million warp instructions per view; issue 63% busy at 14
+// warps per SM, which registers and the block sums in shared memory allow). Of
+// this the exact block test took 3.05 to 2.89 ms, batches of 32 instead of 64
+// with the next rows on their way 2.42, the cheaper staging 2.33. One warp per
+// tile needs many tiles: at 920 tiles 115 against 98 us, at 1840 tiles 134 against
+// 150.
+// ---------------------------------------------------------------------------
+constexpr int kBwdMinTiles = 1408;
+constexpr int kRowPx = 8;      // pixels of a lane
+constexpr int kRowBlocks = 8;  // 8x4 blocks of a tile, one per quad of lanes
+
+// This lane's row of pixels: block (lane / 4) in raster order of the tile's 2 x 4
+// blocks, row lane % 4 of it.
+struct RowInfo {
+    int view, x, y, W, n_in;  // first pixel; how many of the eight lie in the view
+    int64_t pix, plane, color_base;
+    bool vec;                 // all eight lie in the view and 16-byte accesses are aligned
+    float tx0, ty0;           // the tile's first pixel centre
+};
+
+__device__ __forceinline__ RowInfo row_info(const gs_frame& f, int tile) {
+    RowInfo t;
+    t.view = view_of_tile(f, tile);
+    const int local = tile - f.tile_base[t.view];
+    const int tx = local % f.tiles_x[t.view], ty = local / f.tiles_x[t.view];
+    const int lane = threadIdx.x & 31, b = lane >> 2;
+    t.x = tx * kFastTile + (b & 1) * kRowPx;
+    t.y = ty * kFastTile + (b >> 1) * 4 + (lane & 3);
+    t.W = f.width[t.view];
+    const int H = f.height[t.view];
+    t.n_in = t.y < H ? min(max(t.W - t.x, 0), kRowPx) : 0;
+    t.plane = (int64_t)t.W * H;
+    const int64_t pb = f.pix_base[t.view];
+    t.pix = pb + (int64_t)t.y * t.W + t.x;
+    t.color_base = 3 * pb + (int64_t)t.y * t.W + t.x;
+    t.vec = t.n_in == kRowPx && ((t.W | (int)pb) & 3) == 0;
+    t.tx0 = (float)(tx * kFastTile) + 0.5f;
+    t.ty0 = (float)(ty * kFastTile) + 0.5f;
+    return t;
+}
+
+// A row's eight values from or to memory (aligned: two 16-byte accesses).
+template <class T, class V4>
+__device__ __forceinline__ void load_row(const T* __restrict__ p, const RowInfo& t, T (&v)[kRowPx]) {
+    if (t.vec) {
+        const V4 a = reinterpret_cast<const V4*>(p)[0], b = reinterpret_cast<const V4*>(p)[1];
+        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+    } else {
+#pragma unroll
+        for (int i = 0; i < kRowPx; i++)
+            if (i < t.n_in) v[i] = p[i];
+    }
+}
+template <class T, class V4>
+__device__ __forceinline__ void store_row(T* __restrict__ p, const RowInfo& t, const T (&v)[kRowPx]) {
+    if (t.vec) {
+        V4 a, b;
+        a.x = v[0]; a.y = v[1]; a.z = v[2]; a.w = v[3]; b.x = v[4]; b.y = v[5]; b.z = v[6]; b.w = v[7];
+        reinterpret_cast<V4*>(p)[0] = a;
+        reinterpret_cast<V4*>(p)[1] = b;
+    } else {
+#pragma unroll
+        for (int i = 0; i < kRowPx; i++)
+            if (i < t.n_in) p[i] = v[i];
+    }
+}
+
+// Exponents and 2^exponent times opacity at two neighbouring pixels of a row:
+// the rounding sequence e = fma(A dx, dx, fma(C dy, dy, (B dx) dy)) of the
+// tile-8 and tile-32 kernels, the same forward and backward, so that all take
+// identical decisions.
+struct TwoAlphas {
+    f32x2 dx;
+    float e[2], og[2];
+};
+__device__ __forceinline__ TwoAlphas two_alphas(f32x2 x, f32x2 nx, f32x2 A, f32x2 B, f32x2 o, f32x2 dy, f32x2 cy) {
+    TwoAlphas r;
+    r.dx = add2(x, nx);
+    unpack2(fma2(mul2(A, r.dx), r.dx, fma2(cy, dy, mul2(mul2(B, r.dx), dy))), r.e[0], r.e[1]);
+    unpack2(mul2(o, pack2(fast_exp2(r.e[0]), fast_exp2(r.e[1]))), r.og[0], r.og[1]);
+    return r;
+}
+
+struct __align__(16) BwdRow {
+    float nx, ny, A, B;
+    float C, o, r, g;
+    float b, unused[3];
+};
+__device__ __forceinline__ f32x2 load2(const float (&v)[2]) { return pack2(v[0], v[1]); }
+
+template <int CG>
+__device__ __forceinline__ void cp_async(void* smem, const void* gmem) {
+    const uint32_t s = (uint32_t)__cvta_generic_to_shared(smem);
+    if (CG == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s), "l"(gmem) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(s), "l"(gmem), "n"(CG) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// The adjoint by rows. Per pixel and Gaussian, back to front: the transmittance in
+// front of it, dL/dalpha and from it dpow = dL/d(exponent) and the blending
+// weight. A lane sums the nine gradient terms over its row of eight pixels in
+// registers, two shuffles join the block's four rows, and the block's sums wait in
+// shared memory until the batch of 32 list entries is done; then each entry adds
+// its blocks' sums in raster order into its one partial. A pixel the Gaussian does
+// not touch enters with alpha = 0, which leaves its state as it is and adds zeros,
+// so one select per pixel is all the predication there is. The next batch's
+// projected rows are on their way (cp.async) while this one is worked on.
+constexpr int kBwdBatch = 32;
+
+__global__ void __launch_bounds__(32, 16) k_rows_bwd(gs_frame f, gs_config cfg, const uint32_t* __restrict__ range,
+                                                     const uint32_t* __restrict__ src,
+                                                     const uint32_t* __restrict__ emit,
+                                                     const float2* __restrict__ mean2d,
+                                                     const float4* __restrict__ conic_opa,
+                                                     const float4* __restrict__ rgb_depth,
+                                                     const float* __restrict__ t_final,
+                                                     const int32_t* __restrict__ n_contrib,
+                                                     const float* __restrict__ dL_dcolor, float4* __restrict__ part0,
+                                                     float4* __restrict__ part1, float* __restrict__ part2,
+                                                     int64_t capacity, const uint32_t* __restrict__ order,
+                                                     uint32_t* counter, int n_tiles) {
+    __shared__ float2 s_raw_xy[kBwdBatch];  // the next batch's projected rows
+    __shared__ float4 s_raw_co[kBwdBatch];
+    __shared__ float4 s_raw_rgb[kBwdBatch];
+    __shared__ BwdRow s_row[kBwdBatch + 1];  // the last one: a Gaussian that no pixel composites
+    __shared__ uint16_t s_list[kRowBlocks][kBwdBatch + 1];  // row | block sum << 8
+    __shared__ float s_sum[kBwdBatch * kRowBlocks][9];
+    __shared__ int s_item;
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x, blk = lane >> 2;
+    const float inv_log2e = 1.f / kLog2e;
+    const float alpha_min = cfg.alpha_min;
+    if (lane == 0) {
+        BwdRow none = {};
+        none.o = -INFINITY;  // times 2^0: below any alpha_min
+        s_row[kBwdBatch] = none;
+    }
+    for (int tile = next_tile(order, counter, n_tiles, true, &s_item); tile >= 0;
+         tile = next_tile(order, counter, n_tiles, false, &s_item)) {
+        const RowInfo ti = row_info(f, tile);
+        const float py = ti.y + 0.5f;
+        const uint32_t start = range[2 * tile];
+        int nc[kRowPx];
+        f32x2 xs[kRowPx / 2], T2[kRowPx / 2], S2[kRowPx / 2], nr[kRowPx / 2], ng[kRowPx / 2], nb[kRowPx / 2];
+        {
+            float t[kRowPx], r[kRowPx], g[kRowPx], b[kRowPx];
+#pragma unroll
+            for (int i = 0; i < kRowPx; i++) {
+                t[i] = 1.f;
+                r[i] = g[i] = b[i] = 0.f;
+                nc[i] = 0;
+            }
+            if (ti.n_in > 0) {
+                load_row<float, float4>(t_final + ti.pix, ti, t);
+                load_row<int, int4>(n_contrib + ti.pix, ti, nc);
+                load_row<float, float4>(dL_dcolor + ti.color_base, ti, r);
+                load_row<float, float4>(dL_dcolor + ti.color_base + ti.plane, ti, g);
+                load_row<float, float4>(dL_dcolor + ti.color_base + 2 * ti.plane, ti, b);
+            }
+            // S = sum over channels of dL/dC_ch times the colour composited behind the
+            // current Gaussian plus the background seen through T_final: dL/dalpha needs
+            // only this dot product, so one scalar replaces three running colours. The
+            // colour gradients are held negated: with -alpha the packed operations, which
+            // have no negation, then give S, dpow and w dL/dc.
+#pragma unroll
+            for (int p = 0; p < kRowPx / 2; p++) {
+                const int i = 2 * p, j = i + 1;
+                xs[p] = pack2(ti.x + (i + 0.5f), ti.x + (j + 0.5f));
+                T2[p] = pack2(t[i], t[j]);
+                S2[p] = pack2(t[i] * (r[i] * cfg.bg[0] + g[i] * cfg.bg[1] + b[i] * cfg.bg[2]),
+                              t[j] * (r[j] * cfg.bg[0] + g[j] * cfg.bg[1] + b[j] * cfg.bg[2]));
+                nr[p] = pack2(-r[i], -r[j]);
+                ng[p] = pack2(-g[i], -g[j]);
+                nb[p] = pack2(-b[i], -b[j]);
+            }
+        }
+        int nc_blk = nc[0], nc_low = ti.n_in > 0 ? nc[0] : 0x7fffffff;  // the row's (then block's) range
+#pragma unroll
+        for (int i = 1; i < kRowPx; i++) {
+            nc_blk = max(nc_blk, nc[i]);
+            if (i < ti.n_in) nc_low = min(nc_low, nc[i]);
+        }
+        nc_blk = max(nc_blk, __shfl_xor_sync(FULL, nc_blk, 1));
+        nc_blk = max(nc_blk, __shfl_xor_sync(FULL, nc_blk, 2));
+        const int n_list = __reduce_max_sync(FULL, (unsigned)nc_blk);
+        // batches of entries before this position need no test against a pixel's last
+        // contributor (pixels outside the view have none and keep that test on)
+        const int n_plain = ti.n_in == kRowPx ? nc_low : 0;
+        const int n_all = __reduce_min_sync(FULL, (unsigned)n_plain);
+        // pairs past every pixel's last contributor get a zero partial (their
+        // emission slots are summed per Gaussian like all others)
+        const uint32_t len = range[2 * tile + 1] - start;
+        for (uint32_t j = (uint32_t)n_list + lane; j < len; j += 32) {
+            const uint32_t e = emit[start + j];
+            if ((int64_t)e < capacity) {
+                part0[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+                part1[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+                part2[e] = 0.f;
+            }
+        }
+        auto fetch = [&](int q, uint32_t idx) {  // entry q's rows on their way to this lane's places
+            if (q >= 0) {
+                cp_async<8>(&s_raw_xy[lane], mean2d + idx);
+                cp_async<16>(&s_raw_co[lane], conic_opa + idx);
+                cp_async<16>(&s_raw_rgb[lane], rgb_depth + idx);
+            }
+        };
+        uint32_t idx = 0;  // the source row of this lane's entry of the batch after the fetched one
+        if (n_list - 1 - lane >= 0) idx = src[start + n_list - 1 - lane];
+        fetch(n_list - 1 - lane, idx);
+        if (n_list - 1 - 32 - lane >= 0) idx = src[start + n_list - 1 - 32 - lane];
+        for (int end0 = n_list; end0 > 0; end0 -= kBwdBatch) {  // row k is entry end0 - 1 - k
+            const int q = end0 - 1 - lane;
+            const uint32_t em = q >= 0 ? emit[start + q] : 0xffffffffu;
+            cp_async_wait();  // each lane reads only what it fetched itself
+            Entry e;
+            e.blocks = 0;
+            e.plain = true;
+            e.o = 1.f;
+            if (q >= 0) {
+                e = load_entry<2, 4>(s_raw_xy, s_raw_co, s_raw_rgb, lane, ti.tx0, ti.ty0, alpha_min, cfg.alpha_max);
+                float4* w = reinterpret_cast<float4*>(&s_row[lane]);
+                w[0] = make_float4(e.nx, e.ny, e.A, e.B);
+                w[1] = make_float4(e.C, e.o, e.r, e.g);
+                s_row[lane].b = e.b;
+            }
+            fetch(q - kBwdBatch, idx);
+            if (q - 2 * kBwdBatch >= 0) idx = src[start + q - 2 * kBwdBatch];
+#pragma unroll
+            for (int b = 0; b < kRowBlocks; b++)
+                if (q >= __shfl_sync(FULL, nc_blk, 4 * b)) e.blocks &= ~(1u << b);
+            const int mine = __popc(e.blocks);
+            int incl = mine;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(FULL, incl, o);
+                if (lane >= o) incl += u;
+            }
+            const int first = incl - mine;  // this entry's block sums: [first, first + mine)
+            int n_mine = 0, job = first;
+#pragma unroll
+            for (int b = 0; b < kRowBlocks; b++) {
+                const bool hit = (e.blocks >> b) & 1u;
+                const unsigned m = __ballot_sync(FULL, hit);
+                if (hit) {
+                    s_list[b][__popc(m & lanemask_lt())] = (uint16_t)(lane | job << 8);
+                    job++;
+                }
+                if (blk == b) n_mine = __popc(m);
+            }
+            const int n_max = __reduce_max_sync(FULL, (unsigned)n_mine);
+            const bool all = __any_sync(FULL, e.blocks && !e.plain);
+            __syncwarp();
+            // ALL: with the tests that plain Gaussians do without; LIM: with the test against
+            // each pixel's last contributor
+            auto walk = [&](auto all_c, auto lim_c) {
+                constexpr bool ALL = decltype(all_c)::value, LIM = decltype(lim_c)::value;
+                unsigned next = n_mine > 0 ? (unsigned)s_list[blk][0] : (unsigned)kBwdBatch;
+                for (int i = 0; i < n_max; i++) {
+                    const bool live = i < n_mine;
+                    const unsigned ent = next;
+                    next = i + 1 < n_mine ? (unsigned)s_list[blk][i + 1] : (unsigned)kBwdBatch;
+                    const int k = ent & 255u;
+                    const int pos = end0 - 1 - k;
+                    const BwdRow& R = s_row[k];
+                    const float4 q0 = reinterpret_cast<const float4*>(&R)[0], q1 = reinterpret_cast<const float4*>(&R)[1];
+                    const f32x2 nx = both(q0.x), A = both(q0.z), B = both(q0.w), o = both(q1.y);
+                    const f32x2 r2 = both(q1.z), g2 = both(q1.w), b2 = both(R.b);
+                    const float dy = py + q0.y;
+                    const f32x2 dy2 = both(dy), cy2 = both(__fmul_rn(q1.x, dy));
+                    float s0 = 0.f, s1 = 0.f, s3 = 0.f;
+                    f32x2 c6 = 0, c7 = 0, c8 = 0;
+#pragma unroll
+                    for (int p = 0; p < kRowPx / 2; p++) {
+                        const TwoAlphas t = two_alphas(xs[p], nx, A, B, o, dy2, cy2);
+                        // the same decisions as the forward pass: listed before this pixel's last
+                        // contributor, exponent <= 0, alpha >= alpha_min; na = -alpha, or 0. Alpha
+                        // clamped at alpha_max passes no gradient to the exponent or opacity (nog);
+                        // selects (not products with 0) keep a non-finite 2^e outside the Gaussian
+                        // out of the sums.
+                        float na[2], nog[2], m[2], dx[2], d[2];
+#pragma unroll
+                        for (int h = 0; h < 2; h++) {
+                            const float alpha = ALL ? fminf(cfg.alpha_max, t.og[h]) : t.og[h];
+                            bool in = alpha >= alpha_min;
+                            if (LIM) in = in && pos < nc[2 * p + h];
+                            if (ALL) in = in && !(t.e[h] > 0.f);
+                            na[h] = in ? -alpha : 0.f;
+                            nog[h] = ALL ? (in && t.og[h] < cfg.alpha_max ? -t.og[h] : 0.f) : na[h];
+                        }
+                        unpack2(add2(load2(na), both(1.f)), m[0], m[1]);
+                        const f32x2 inv = pack2(fast_rcp(m[0]), fast_rcp(m[1]));
+                        const f32x2 ngc = fma2(nb[p], b2, fma2(nr[p], r2, mul2(ng[p], g2)));
+                        T2[p] = mul2(T2[p], inv);  // transmittance in front of this Gaussian (1/1 = 1 keeps it)
+                        const f32x2 nw = mul2(load2(na), T2[p]);
+                        // -dL/dalpha = S / (1 - alpha) - T sum_ch dL/dC_ch c_ch
+                        const f32x2 ndal = fma2(T2[p], ngc, mul2(S2[p], inv));
+                        S2[p] = fma2(nw, ngc, S2[p]);
+                        unpack2(mul2(ndal, load2(nog)), d[0], d[1]);  // d alpha / d(natural exponent) dL/dalpha
+                        unpack2(t.dx, dx[0], dx[1]);
+#pragma unroll
+                        for (int h = 0; h < 2; h++) {
+                            s0 += d[h];
+                            const float t1 = __fmul_rn(d[h], dx[h]);
+                            s1 = __fadd_rn(s1, t1);
+                            s3 = __fmaf_rn(t1, dx[h], s3);
+                        }
+                        c6 = fma2(nw, nr[p], c6);
+                        c7 = fma2(nw, ng[p], c7);
+                        c8 = fma2(nw, nb[p], c8);
+                    }
+                    // The block's sums, rows (0 + 1) + (2 + 3): in the first step the lanes of
+                    // rows 0 and 2 keep the terms of dx and dy, those of rows 1 and 3 the others,
+                    // in the second each lane keeps two (three in row 0) and finishes them.
+                    float u, v, k0, k1, k2, k3, k4;
+                    {
+                        const bool odd = lane & 1;
+                        const float dy1 = __fmul_rn(dy, s0);
+                        auto part = [&](float keep_even, float keep_odd) {
+                            const float give = odd ? keep_even : keep_odd;
+                            return __fadd_rn(odd ? keep_odd : keep_even, __shfl_xor_sync(FULL, give, 1));
+                        };
+                        unpack2(c6, u, v);
+                        const float s6 = u + v;
+                        unpack2(c7, u, v);
+                        const float s7 = u + v;
+                        unpack2(c8, u, v);
+                        const float s8 = u + v;
+                        k0 = part(s1, __fmul_rn(dy, dy1));
+                        k1 = part(dy1, s6);
+                        k2 = part(s3, s7);
+                        k3 = part(__fmul_rn(dy, s1), s8);
+                        k4 = __fadd_rn(s0, __shfl_xor_sync(FULL, s0, 1));
+                    }
+                    {
+                        const bool low = lane & 2;  // rows 2 and 3
+                        const float g0 = low ? k0 : k2, g1 = low ? k1 : k3;
+                        u = __fadd_rn(low ? k2 : k0, __shfl_xor_sync(FULL, g0, 2));
+                        v = __fadd_rn(low ? k3 : k1, __shfl_xor_sync(FULL, g1, 2));
+                        k4 = __fadd_rn(k4, __shfl_xor_sync(FULL, k4, 2));
+                    }
+                    // row 0: dx, dy, sum(dpow); row 1: dy dy, red; row 2: dx dx, dx dy; row 3: green, blue
+                    if (live) {
+                        float* out = s_sum[ent >> 8] + 2 * (lane & 3);
+                        const float a = q0.z, b = q0.w, cc = q1.x;
+                        const float m0 = -inv_log2e * (2.f * a * u + b * v), m1 = -inv_log2e * (b * u + 2.f * cc * v);
+                        const bool row0 = (lane & 3) == 0;
+                        out[0] = row0 ? m0 : u;
+                        out[1] = row0 ? m1 : v;
+                        if (row0) out[8] = k4;
+                    }
+                }
+            };
+            if (all) walk(BoolC<true>{}, BoolC<true>{});
+            else if (end0 > n_all) walk(BoolC<false>{}, BoolC<true>{});
+            else walk(BoolC<false>{}, BoolC<false>{});
+            __syncwarp();
+            if ((int64_t)em < capacity) {  // (no entry: past any capacity)
+                float a[9];
+#pragma unroll
+                for (int c = 0; c < 9; c++) a[c] = 0.f;
+                for (int j = first; j < first + mine; j++)
+#pragma unroll
+                    for (int c = 0; c < 9; c++) a[c] += s_sum[j][c];
+                // sum of dalpha G = sum of dalpha (o G) / o
+                part0[em] = make_float4(a[0], a[1], -0.5f * a[4], -a[5]);
+                part1[em] = make_float4(-0.5f * a[2], e.o > 0.f ? a[8] / e.o : 0.f, a[3], a[6]);
+                part2[em] = a[7];
+            }
+            __syncwarp();  // rows, lists and sums are rewritten by the next batch
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
 // Launch configurations (the autotuner picks among these)
 // ---------------------------------------------------------------------------
 struct RenderLaunch {
@@ -461,7 +1169,15 @@ struct RenderLaunch {
     int threads;
 };
 
-static RenderLaunch pick_fwd(int tile, int batch, bool depth = false, bool count = false) {
+static RenderLaunch pick_fwd(int tile, int batch, int n_tiles, bool depth = false, bool count = false) {
+#define GS_BLOCKS(B)                                                    \
+    if (tile == kFastTile && n_tiles >= kFwdMinTiles && batch == B)     \
+        return {count   ? (const void*)k_blocks_fwd<B, false, true>     \
+                : depth ? (const void*)k_blocks_fwd<B, true>            \
+                        : (const void*)k_blocks_fwd<B, false>,          \
+                kFwdThreads};
+    GS_BLOCKS(64) GS_BLOCKS(128) GS_BLOCKS(256)
+#undef GS_BLOCKS
 #define GS_FWD(T, B)                                                                     \
     if (tile == T && batch == B)                                                         \
         return {count   ? (const void*)k_render_fwd<T, B, false, true>                   \
@@ -475,7 +1191,10 @@ static RenderLaunch pick_fwd(int tile, int batch, bool depth = false, bool count
     return {nullptr, 0};
 }
 
-static RenderLaunch pick_bwd(int tile, int batch) {
+static RenderLaunch pick_bwd(int tile, int batch, int n_tiles) {
+    // k_rows_bwd has one batch size (its block sums take most of the shared memory)
+    if (tile == kFastTile && n_tiles >= kBwdMinTiles && (batch == 32 || batch == 64 || batch == 128))
+        return {(const void*)k_rows_bwd, 32};
 #define GS_BWD(T, B) if (tile == T && batch == B) return {(const void*)k_render_bwd<T, B>, T * T};
     GS_BWD(8, 64) GS_BWD(8, 128) GS_BWD(8, 256)
     GS_BWD(16, 32) GS_BWD(16, 64) GS_BWD(16, 128)
@@ -484,7 +1203,9 @@ static RenderLaunch pick_bwd(int tile, int batch) {
     return {nullptr, 0};
 }
 
-static int default_fwd_batch(int tile) { return tile == 8 ? 128 : 256; }
+static int default_fwd_batch(int tile, int n_tiles) {
+    return tile == 8 || (tile == kFastTile && n_tiles >= kFwdMinTiles) ? 128 : 256;
+}
 static int default_bwd_batch(int tile) { return tile == 32 ? 32 : tile == 16 ? 64 : 128; }
 
 static int launch(const RenderLaunch& L, int n_tiles, bool persistent, void** args, cudaStream_t s) {
@@ -502,8 +1223,8 @@ static int launch(const RenderLaunch& L, int n_tiles, bool persistent, void** ar
 }
 
 bool render_batch_supported(int tile, int fwd_batch, int bwd_batch) {
-    return pick_fwd(tile, fwd_batch ? fwd_batch : default_fwd_batch(tile)).fn != nullptr &&
-           pick_bwd(tile, bwd_batch ? bwd_batch : default_bwd_batch(tile)).fn != nullptr;
+    return pick_fwd(tile, fwd_batch ? fwd_batch : default_fwd_batch(tile, 0), 0).fn != nullptr &&
+           pick_bwd(tile, bwd_batch ? bwd_batch : default_bwd_batch(tile), 0).fn != nullptr;
 }
 
 }  // namespace gs
@@ -537,8 +1258,8 @@ static int render_fwd_impl(const gs_projected* p, const gs_pairs* pairs, const g
     uint32_t* counter = persistent ? (uint32_t*)ws : nullptr;
     const uint32_t* order = persistent || ordered ? pairs->order : nullptr;
     if (persistent) cudaMemsetAsync(counter, 0, sizeof(uint32_t), s);
-    const RenderLaunch L = pick_fwd(cfg->tile, cfg->fwd_batch ? cfg->fwd_batch : default_fwd_batch(cfg->tile),
-                                    out->depth != nullptr && !counts, counts != nullptr);
+    const RenderLaunch L = pick_fwd(cfg->tile, cfg->fwd_batch ? cfg->fwd_batch : default_fwd_batch(cfg->tile, n_tiles),
+                                    n_tiles, out->depth != nullptr && !counts, counts != nullptr);
     gs_frame fv = *f;
     gs_config cv = *cfg;
     const uint32_t* range = pairs->range;
@@ -580,7 +1301,7 @@ int launch_render_bwd(const gs_projected* p, const gs_pairs* pairs, const gs_fra
     const uint32_t* order = persistent || ordered ? pairs->order : nullptr;
     if (!persistent) counter = nullptr;
     if (persistent) cudaMemsetAsync(counter, 0, sizeof(uint32_t), s);
-    const RenderLaunch L = pick_bwd(cfg->tile, cfg->bwd_batch ? cfg->bwd_batch : default_bwd_batch(cfg->tile));
+    const RenderLaunch L = pick_bwd(cfg->tile, cfg->bwd_batch ? cfg->bwd_batch : default_bwd_batch(cfg->tile), n_tiles);
     gs_frame fv = *f;
     gs_config cv = *cfg;
     const uint32_t* range = pairs->range;
