@@ -104,6 +104,12 @@ size_t scan_workspace_bytes(int64_t n_max);
 // Device-wide exclusive scan of n uint32 values; total (device) gets the sum.
 void scan_exclusive_u32(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* total, void* ws, cudaStream_t s);
 
+// The same of the words' numbers of set bits, in one launch (single-pass, decoupled
+// look-back). ws: scan_popcounts_words(n) words, 8-byte aligned, cleared by an
+// earlier launch. Returns the device word with 0, or GS_ERR_TIMEOUT from a bounded wait.
+size_t scan_popcounts_words(int64_t n);
+int32_t* scan_popcounts(const uint32_t* words, uint32_t* out, int64_t n, uint32_t* total, uint32_t* ws, cudaStream_t s);
+
 // Stable LSD radix sort of (uint32 key, uint32 value) pairs on key bits
 // [0, bits), 8 bits per pass. The pair count is min(n_max, *n_dev). Buffers
 // (ka, va) hold the input; (kb, vb) are the alternates. With va_is_position

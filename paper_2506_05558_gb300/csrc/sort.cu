@@ -556,6 +556,19 @@ static void scan_single(Load load, uint32_t* out, int64_t n_max, const uint32_t*
     count_launch();
 }
 
+struct LoadPopcount {
+    const uint32_t* words;
+    __device__ uint32_t operator()(int64_t i) const { return (uint32_t)__popc(words[i]); }
+};
+
+size_t scan_popcounts_words(int64_t n) { return 64 + 2 * ceil_div(n, kScanTile); }
+
+int32_t* scan_popcounts(const uint32_t* words, uint32_t* out, int64_t n, uint32_t* total, uint32_t* ws, cudaStream_t s) {
+    int32_t* err = (int32_t*)ws + 32;
+    scan_single(LoadPopcount{words}, out, n, nullptr, total, (ScanCtl*)ws, (uint64_t*)(ws + 64), err, s);
+    return err;
+}
+
 // Digit counts of every pass in one read of the keys (shared-memory atomics
 // into per-warp sub-histograms), then, in the last CTA to finish, their
 // exclusive sums: the global start of each digit. Also zeroes the first
