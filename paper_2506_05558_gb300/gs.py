@@ -308,12 +308,12 @@ class Projected:
     n_tiles: torch.Tensor
 
     @staticmethod
-    def alloc(items, device="cuda") -> "Projected":
-        return Projected(torch.zeros((items, 2), dtype=torch.float32, device=device),
-                         torch.zeros((items, 4), dtype=torch.float32, device=device),
-                         torch.zeros((items, 4), dtype=torch.float32, device=device),
-                         torch.zeros((items, 4), dtype=torch.int16, device=device),
-                         torch.zeros((items,), dtype=torch.int32, device=device))
+    def alloc(items, device="cuda", new=torch.zeros) -> "Projected":
+        return Projected(new((items, 2), dtype=torch.float32, device=device),
+                         new((items, 4), dtype=torch.float32, device=device),
+                         new((items, 4), dtype=torch.float32, device=device),
+                         new((items, 4), dtype=torch.int16, device=device),
+                         new((items,), dtype=torch.int32, device=device))
 
     def c(self) -> gs_projected:
         return gs_projected(_ptr(self.mean2d), _ptr(self.conic_opa), _ptr(self.rgb_depth), _ptr(self.rect),
@@ -335,11 +335,10 @@ class Pairs:
         return int(self.src.shape[0])
 
     @staticmethod
-    def alloc(items, n_tiles_total, capacity, device="cuda", with_order=True) -> "Pairs":
-        u32 = lambda k: torch.zeros((k,), dtype=torch.int32, device=device)
+    def alloc(items, n_tiles_total, capacity, device="cuda", with_order=True, new=torch.zeros) -> "Pairs":
+        u32 = lambda k: new((k,), dtype=torch.int32, device=device)
         return Pairs(u32(max(capacity, 1)), u32(max(capacity, 1)), u32(max(items, 1)), u32(2 * n_tiles_total),
-                     torch.zeros((1,), dtype=torch.int64, device=device),
-                     torch.zeros((1,), dtype=torch.int32, device=device),
+                     new((1,), dtype=torch.int64, device=device), new((1,), dtype=torch.int32, device=device),
                      u32(max(n_tiles_total, 1)) if with_order else None)
 
     def c(self) -> gs_pairs:
@@ -355,11 +354,11 @@ class Image:
     depth: torch.Tensor | None = None  # depth integral, written only when present
 
     @staticmethod
-    def alloc(n_pix, device="cuda", with_depth=False) -> "Image":
-        return Image(torch.zeros((3 * n_pix,), dtype=torch.float32, device=device),
-                     torch.zeros((n_pix,), dtype=torch.float32, device=device),
-                     torch.zeros((n_pix,), dtype=torch.int32, device=device),
-                     torch.zeros((n_pix,), dtype=torch.float32, device=device) if with_depth else None)
+    def alloc(n_pix, device="cuda", with_depth=False, new=torch.zeros) -> "Image":
+        return Image(new((3 * n_pix,), dtype=torch.float32, device=device),
+                     new((n_pix,), dtype=torch.float32, device=device),
+                     new((n_pix,), dtype=torch.int32, device=device),
+                     new((n_pix,), dtype=torch.float32, device=device) if with_depth else None)
 
     def c(self) -> gs_image:
         return gs_image(_ptr(self.color), _ptr(self.t_final), _ptr(self.n_contrib), _ptr(self.depth))
@@ -374,9 +373,9 @@ class Grads:
     visible: torch.Tensor
 
     @staticmethod
-    def alloc(n, device="cuda") -> "Grads":
-        z = lambda k: torch.zeros((n, k), dtype=torch.float32, device=device)
-        return Grads(z(4), z(4), z(4), z(48), torch.zeros((n,), dtype=torch.uint8, device=device))
+    def alloc(n, device="cuda", new=torch.zeros) -> "Grads":
+        z = lambda k: new((n, k), dtype=torch.float32, device=device)
+        return Grads(z(4), z(4), z(4), z(48), new((n,), dtype=torch.uint8, device=device))
 
     def c(self) -> gs_grads:
         return gs_grads(_ptr(self.mean_opa), _ptr(self.scale), _ptr(self.quat), _ptr(self.sh), _ptr(self.visible))

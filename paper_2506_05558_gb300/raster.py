@@ -16,7 +16,10 @@ from . import gs
 
 
 class Rasterizer:
-    def __init__(self, n: int, sizes, capacity: int, cfg: gs.gs_config | None = None, device="cuda"):
+    def __init__(self, n: int, sizes, capacity: int, cfg: gs.gs_config | None = None, device="cuda",
+                 lazy: bool = False):
+        """lazy: the buffers are made by forward_fit, each while the stage before runs, and
+        not filled: for a caller that reads only what the stages have written."""
         self.n = int(n)
         self.sizes = list(sizes)
         self.n_views = len(self.sizes)
@@ -26,20 +29,39 @@ class Rasterizer:
         self.n_pix = int(self.f.pix_base[self.n_views])
         self.n_tiles = int(self.f.tile_base[self.n_views])
         self.device = device
-        self.proj = gs.Projected.alloc(self.items, device)
-        self.img = gs.Image.alloc(self.n_pix, device)
-        self.ws_render = gs.workspace(gs.gs_render_workspace_size(self.f), device)
-        self.grads = gs.Grads.alloc(self.n, device)
-        self.dpose = torch.zeros((self.n_views, 6), dtype=torch.float32, device=device)
-        self.set_capacity(capacity)
+        self.new = torch.empty if lazy else torch.zeros
+        self.capacity = max(int(capacity), 1)
+        if not lazy:
+            self._alloc_projected()
+            self._alloc_image()
+            self._alloc_gradients()
+            self.set_capacity(capacity)
+
+    def _alloc_projected(self):
+        self.proj = gs.Projected.alloc(self.items, self.device, new=self.new)
+
+    def _alloc_image(self):
+        self.img = gs.Image.alloc(self.n_pix, self.device, new=self.new)
+        self.ws_render = gs.workspace(gs.gs_render_workspace_size(self.f), self.device)
+
+    def _alloc_gradients(self):
+        # cfg.accumulate adds to the first contents
+        self.grads = gs.Grads.alloc(self.n, self.device, new=torch.zeros if self.cfg.accumulate else self.new)
+        self.dpose = self.new((self.n_views, 6), dtype=torch.float32, device=self.device)
+
+    def _alloc_pairs(self):
+        # the tile work order is only read by schedules 1 and 2; without it gs_sort skips that sort
+        self.pairs = gs.Pairs.alloc(self.items, self.n_tiles, self.capacity, self.device,
+                                    with_order=self.cfg.schedule in (1, 2), new=self.new)
+        self.ws_sort = gs.workspace(gs.gs_sort_workspace_size(self.n, self.f, self.capacity), self.device)
+
+    def _alloc_bwd_workspace(self):
+        self.ws_bwd = gs.workspace(gs.gs_backward_workspace_size(self.n, self.f, self.capacity), self.device)
 
     def set_capacity(self, capacity: int):
         self.capacity = max(int(capacity), 1)
-        # the tile work order is only read by schedules 1 and 2; without it gs_sort skips that sort
-        self.pairs = gs.Pairs.alloc(self.items, self.n_tiles, self.capacity, self.device,
-                                    with_order=self.cfg.schedule in (1, 2))
-        self.ws_sort = gs.workspace(gs.gs_sort_workspace_size(self.n, self.f, self.capacity), self.device)
-        self.ws_bwd = gs.workspace(gs.gs_backward_workspace_size(self.n, self.f, self.capacity), self.device)
+        self._alloc_pairs()
+        self._alloc_bwd_workspace()
 
     # -- stages ---------------------------------------------------------------
     def forward(self, g: gs.Gaussians, cams: torch.Tensor, stream=None):
@@ -47,6 +69,33 @@ class Rasterizer:
         gs.gs_sort(self.proj, self.n, self.f, self.pairs, self.ws_sort, stream)
         gs.gs_render_fwd(self.proj, self.pairs, self.f, self.cfg, self.img, self.ws_render, stream)
         return self.img
+
+    def forward_fit(self, g: gs.Gaussians, cams: torch.Tensor, slack: float = 1.25):
+        """forward() of a lazy rasteriser with room for every pair: the host waits for the
+        sort's pair count while the render runs, and sorts and renders again with a
+        grown pair buffer (slack x the count) where it did not fit."""
+        self._alloc_projected()
+        gs.gs_project(g, cams, self.f, self.cfg, self.proj)
+        count = torch.empty((1,), dtype=torch.int64, pin_memory=True)
+        sorted_ = torch.cuda.Event()
+        self._alloc_pairs()
+        gs.gs_sort(self.proj, self.n, self.f, self.pairs, self.ws_sort)
+        count.copy_(self.pairs.count, non_blocking=True)
+        sorted_.record()
+        self._alloc_image()
+        while True:
+            gs.gs_render_fwd(self.proj, self.pairs, self.f, self.cfg, self.img, self.ws_render)
+            if not hasattr(self, "grads"):
+                self._alloc_gradients()
+                self._alloc_bwd_workspace()
+            sorted_.synchronize()
+            p = int(count[0])
+            if p <= self.capacity:
+                return self.img
+            self.set_capacity(int(math.ceil(p * slack)) + 1024)
+            gs.gs_sort(self.proj, self.n, self.f, self.pairs, self.ws_sort)
+            count.copy_(self.pairs.count, non_blocking=True)
+            sorted_.record()
 
     def backward(self, g: gs.Gaussians, cams: torch.Tensor, dL_dcolor: torch.Tensor, d_proj=None, stream=None):
         gs.gs_render_bwd(g, cams, self.proj, self.pairs, self.f, self.cfg, self.img, dL_dcolor, self.grads,
