@@ -9,11 +9,14 @@
 // operands: forward Z = H W^T (A = H, B = W), input gradient dH = dZ W (A = dZ,
 // B = W^T), weight gradient dW = dZ^T H (A = dZ^T, B = H^T). Elementwise work
 // (bias, GELU, its derivative, the loss, the casts) sits in small kernels
-// around the GEMMs; partial sums over patches are reduced in a fixed order.
+// around the GEMMs; partial sums over patches are reduced in a fixed order. On the
+// tcgen05 path with a 16-byte aligned image a training step is three launches that keep
+// the products' and sums' order (mlp_tc.cu).
 #include <cuda_bf16.h>
 
 #include "common.cuh"
 #include "mlp_gemm.cuh"
+#include "mlp_train.cuh"
 
 namespace gs {
 
@@ -207,17 +210,24 @@ __global__ void k_split_sum(const float* __restrict__ part, int S, int R, int C,
     out[i] = s;
 }
 
-__global__ void k_sum_partials(const float* __restrict__ p, int n, float* __restrict__ out) {
+// The sum of 256 strided sums by a tree over them (any block of NT threads, NT <= 256).
+template <int NT>
+__device__ __forceinline__ void sum_partials(const float* __restrict__ p, int n, float* __restrict__ out) {
     __shared__ float s[256];
-    float a = 0.f;
-    for (int i = threadIdx.x; i < n; i += 256) a += p[i];
-    s[threadIdx.x] = a;
+    for (int t = threadIdx.x; t < 256; t += NT) {
+        float a = 0.f;
+        for (int i = t; i < n; i += 256) a += p[i];
+        s[t] = a;
+    }
     __syncthreads();
     for (int h = 128; h > 0; h >>= 1) {
-        if (threadIdx.x < h) s[threadIdx.x] += s[threadIdx.x + h];
+        for (int t = threadIdx.x; t < h; t += NT) s[t] += s[t + h];
         __syncthreads();
     }
     if (threadIdx.x == 0) *out = s[0];
+}
+__global__ void k_sum_partials(const float* __restrict__ p, int n, float* __restrict__ out) {
+    sum_partials<256>(p, n, out);
 }
 
 // The four layers' casts in one launch: thread i of the concatenated padded
@@ -247,21 +257,92 @@ struct AdamAll {
     float *p[8], *m[8], *v[8];
     int64_t seg_end[8];
 };
+__device__ __forceinline__ void adam_one(const AdamAll& a, int k, int64_t j, float gi, float lr, float b1, float b2,
+                                         float eps, float t) {
+    const float bc1 = 1.f - powf(b1, t), bc2 = 1.f - powf(b2, t);
+    const float mi = b1 * a.m[k][j] + (1.f - b1) * gi;
+    const float vi = b2 * a.v[k][j] + (1.f - b2) * gi * gi;
+    a.m[k][j] = mi;
+    a.v[k][j] = vi;
+    a.p[k][j] -= lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
+}
 __global__ void k_mlp_adam_all(AdamAll a, const float* __restrict__ g, float lr, float b1, float b2, float eps,
                                int32_t step, const int32_t* __restrict__ step_dev) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int k = 0;
     while (k < 8 && i >= a.seg_end[k]) k++;
     if (k == 8) return;
-    const int64_t j = i - (k > 0 ? a.seg_end[k - 1] : 0);
-    const float t = step_dev ? (float)*step_dev : (float)step;
-    const float bc1 = 1.f - powf(b1, t), bc2 = 1.f - powf(b2, t);
-    const float gi = g[i];
-    const float mi = b1 * a.m[k][j] + (1.f - b1) * gi;
-    const float vi = b2 * a.v[k][j] + (1.f - b2) * gi * gi;
-    a.m[k][j] = mi;
-    a.v[k][j] = vi;
-    a.p[k][j] -= lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
+    adam_one(a, k, i - (k > 0 ? a.seg_end[k - 1] : 0), g[i], lr, b1, b2, eps,
+             step_dev ? (float)*step_dev : (float)step);
+}
+
+// Gradients and Adam after k_mlp_backward_tc: each parameter's shares are added in split
+// order, written to `grads` (null: not) and the parameter stepped (a.p[0] null: not). A
+// block takes 128 words of a split's shares, 8 inputs of 16 neurons (the shares
+// have neurons side by side, the parameters inputs: 64-byte and 32-byte runs; 128
+// neurons of one input took twice as long for the scattered Adam state), and copies 36
+// splits of them to shared memory while it adds the 36 before. The last block adds the
+// loss (as k_sum_partials).
+constexpr int kRedThreads = 128, kRedRows = 36, kRedPitch = 20;  // words from input to input: no bank conflicts
+__global__ void __launch_bounds__(kRedThreads) k_mlp_reduce(AdamAll a, const float* __restrict__ part, int splits,
+                                                            const float* __restrict__ loss_part, float* __restrict__ loss,
+                                                            float* __restrict__ grads, float lr, float b1, float b2,
+                                                            float eps, int32_t step,
+                                                            const int32_t* __restrict__ step_dev) {
+    __shared__ __align__(16) float s_v[2][kRedRows][8 * kRedPitch];
+    if (blockIdx.x == gridDim.x - 1) {
+        sum_partials<kRedThreads>(loss_part, splits, loss);
+        return;
+    }
+    // first word of each of the block's 8 runs of 16: base + run * pitch
+    const int at = blockIdx.x * kRedThreads;
+    const int l = at >= kMlpPartB0 ? 4 : at >= kMlpPartW3 ? 3 : at >= kMlpPartW2 ? 2 : at >= kMlpPartW1 ? 1 : 0;
+    const int n_out = l == 3 ? kOutPad : l == 4 ? 16 : kHid;  // neurons per input; the biases are one run after another
+    const int first = l == 4 ? kMlpPartB0 : l == 3 ? kMlpPartW3 : l == 2 ? kMlpPartW2 : l == 1 ? kMlpPartW1 : kMlpPartW0;
+    const int tile = (at - first) / kRedThreads, across = n_out / 16;
+    const int c0 = tile / across * 8, n0 = tile % across * 16;
+    const float* src = part + first + c0 * n_out + n0;
+    auto fetch = [&](int z0, int buf) {
+        const int n = min(kRedRows, splits - z0) * 32;
+        for (int q = threadIdx.x; q < n; q += kRedThreads) {
+            const int z = q / 32, run = q / 4 % 8, e = q % 4 * 4;
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(
+                             (uint32_t)__cvta_generic_to_shared(&s_v[buf][z][run * kRedPitch + e])),
+                         "l"(src + (int64_t)(z0 + z) * kMlpPart + run * n_out + e)
+                         : "memory");
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+    fetch(0, 0);
+    const int c = threadIdx.x % 8, n = threadIdx.x / 8;
+    float g = 0.f;
+    for (int z0 = 0, buf = 0; z0 < splits; z0 += kRedRows, buf ^= 1) {
+        if (z0 + kRedRows < splits) {
+            fetch(z0 + kRedRows, buf ^ 1);
+            asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+        }
+        __syncthreads();
+        const int rows = min(kRedRows, splits - z0);
+#pragma unroll 4
+        for (int z = 0; z < rows; z++) g += s_v[buf][z][c * kRedPitch + n];
+        __syncthreads();
+    }
+    // the parameter: tensor k, element j
+    int k, j;
+    if (l == 4) {  // block = layer
+        j = c * 16 + n;
+        k = 2 * (c0 / 8) + 1;
+        if (j >= (k == 7 ? kOut : kHid)) return;
+    } else {
+        const int n_in = l == 0 ? kIn : kHid;
+        if (c0 + c >= n_in || n0 + n >= (l == 3 ? kOut : kHid)) return;
+        j = (n0 + n) * n_in + c0 + c;
+        k = 2 * l;
+    }
+    if (grads) grads[(k > 0 ? a.seg_end[k - 1] : 0) + j] = g;
+    if (a.p[0]) adam_one(a, k, j, g, lr, b1, b2, eps, step_dev ? (float)*step_dev : (float)step);
 }
 
 // ---------------------------------------------------------------------------
@@ -312,7 +393,7 @@ static MlpWs carve_mlp(char* base, size_t cap, int64_t M, size_t* used) {
     w.dZf = c.take<float>(Mp * kHid);
     w.dY = c.take<float>(Mp * kOutPad);
     w.splits = ceil_div(Mp, kSplitK);
-    w.part = c.take<float>((size_t)w.splits * kHid * kInPad);
+    w.part = c.take<float>((size_t)w.splits * kMlpPart);
     w.nb_loss = ceil_div(Mp, 256);
     w.loss_part = c.take<float>(w.nb_loss);
     w.grad = c.take<float>(n_params_total());
@@ -322,10 +403,6 @@ static MlpWs carve_mlp(char* base, size_t cap, int64_t M, size_t* used) {
 
 int mlp_forward_fused(const float* const* w, const float* const* b, const float* image, int W, int H, float* out,
                       cudaStream_t s);
-int mlp_train_forward_fused(const float* const* w, const float* const* b, const float* image, int W, int H,
-                            __nv_bfloat16* Xt, float* const* Z, __nv_bfloat16* const* Ht, float* Z3, int64_t Mp,
-                            cudaStream_t s);
-
 struct MlpPtrs {
     float* w[4];
     float* b[4];
@@ -369,16 +446,6 @@ static int mlp_forward(const MlpPtrs& P, const float* image, int W, int H, const
                        const float* targets, float w_depth, float w_scale, float* out, cudaStream_t s) {
     const int64_t M = w.M, Mp = w.Mp;
     cast_weights(P, w, s);
-    if (path == 1 && targets && ((uintptr_t)image & 15) == 0) {
-        // training forward on the tensor cores in one persistent kernel (weights resident in shared
-        // memory), writing the tensors the backward reads; then the loss as below
-        int rc = mlp_train_forward_fused(P.w, P.b, image, W, H, w.Xt, w.Z, w.Ht, w.Z[3], Mp, s);
-        if (rc != GS_OK) return rc;
-        k_mlp_loss<<<(unsigned)w.nb_loss, 256, 0, s>>>(w.Z[3], P.b[3], targets, M, Mp, w_depth, w_scale, out, w.dY,
-                                                        w.dZ4, w.dZ4t, w.loss_part);
-        count_launch();
-        return GS_OK;
-    }
     k_mlp_features<<<dim3((unsigned)ceil_div(kInPad, 32), (unsigned)ceil_div(Mp, 32)), dim3(32, 8), 0, s>>>(
         image, W, H, M, Mp, w.X, w.Xt);
     count_launch();
@@ -497,6 +564,34 @@ extern "C" int gs_mlp_train_step(const gs_mlp_params* p, const gs_mlp_params* m,
         return GS_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     const MlpPtrs P = ptrs(p);
+    AdamAll a{};  // no pointers: no update
+    int64_t off = 0;
+    for (int l = 0; l < 4; l++) {
+        off += (int64_t)kRv[l] * kCv[l];
+        a.seg_end[2 * l] = off;
+        off += kRv[l];
+        a.seg_end[2 * l + 1] = off;
+        if (m) {
+            const MlpPtrs Pm = ptrs(m), Pv = ptrs(v);
+            a.p[2 * l] = P.w[l]; a.m[2 * l] = Pm.w[l]; a.v[2 * l] = Pv.w[l];
+            a.p[2 * l + 1] = P.b[l]; a.m[2 * l + 1] = Pm.b[l]; a.v[2 * l + 1] = Pv.b[l];
+        }
+    }
+    if (cfg->tensor_path == 1 && ((uintptr_t)image & 15) == 0) {
+        // three launches: forward, loss and backward per split of patches, and the sums with Adam
+        // (1080p, 32400 patches: 128 us, of which the forward 57; 22 launches of the product chain took 457)
+        const MlpTrainBufs t{w.Xt, {w.Z[0], w.Z[1], w.Z[2]}, {w.Ht[0], w.Ht[1], w.Ht[2]}, w.Z[3],
+                             {w.Wt[1], w.Wt[2], w.Wt[3]}, w.part, w.loss_part};
+        rc = mlp_train_fused(P.w, P.b, image, width, height, t, w.M, w.Mp, targets, cfg->w_depth, cfg->w_scale, out, s);
+        if (rc != GS_OK) return rc;
+        static_assert(kMlpPart % kRedThreads == 0 && kMlpPartB1 - kMlpPartB0 == kRedThreads);
+        k_mlp_reduce<<<kMlpPart / kRedThreads + 1, kRedThreads, 0, s>>>(a, w.part, (int)w.splits, w.loss_part, loss, grads,
+                                                                  cfg->lr, cfg->beta1, cfg->beta2, cfg->eps, step,
+                                                                  step_dev);
+        count_launch();
+        GS_CUDA_CHECK_LAUNCH();
+        return GS_OK;
+    }
     rc = mlp_forward(P, image, width, height, w, cfg->tensor_path, targets, cfg->w_depth, cfg->w_scale, out, s);
     if (rc != GS_OK) return rc;
     k_sum_partials<<<1, 256, 0, s>>>(w.loss_part, (int)w.nb_loss, loss);
@@ -507,18 +602,6 @@ extern "C" int gs_mlp_train_step(const gs_mlp_params* p, const gs_mlp_params* m,
         cudaMemcpyAsync(grads, w.grad, sizeof(float) * n_params_total(), cudaMemcpyDeviceToDevice, s);
     }
     if (m) {
-        const MlpPtrs Pm = ptrs(m), Pv = ptrs(v);
-        AdamAll a;
-        int64_t off = 0;
-        for (int l = 0; l < 4; l++) {
-            const int64_t nw = (int64_t)kRv[l] * kCv[l], nbias = kRv[l];
-            a.p[2 * l] = P.w[l]; a.m[2 * l] = Pm.w[l]; a.v[2 * l] = Pv.w[l];
-            a.p[2 * l + 1] = P.b[l]; a.m[2 * l + 1] = Pm.b[l]; a.v[2 * l + 1] = Pv.b[l];
-            off += nw;
-            a.seg_end[2 * l] = off;
-            off += nbias;
-            a.seg_end[2 * l + 1] = off;
-        }
         k_mlp_adam_all<<<(unsigned)ceil_div(off, 256), 256, 0, s>>>(a, w.grad, cfg->lr, cfg->beta1, cfg->beta2,
                                                                      cfg->eps, step, step_dev);
         count_launch();
