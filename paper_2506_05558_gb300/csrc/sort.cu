@@ -1216,6 +1216,238 @@ __global__ void k_copy_u32(const uint32_t* __restrict__ a, uint32_t* __restrict_
     if (i < n) b[i] = a[i];
 }
 
+// ---------------------------------------------------------------------------
+// The whole of gs_sort in one CTA, for frames whose items, pairs and tiles fit its
+// shared memory: offsets and compaction, depth sort (8-bit passes in shared memory, those
+// whose digit all keys share skipped), pairs in depth order, one counting pass over the
+// tiles that writes the lists, ranges and work order. 1000 items, 2000 pairs, 16 tiles:
+// 18 us against 51 for the general path's eleven launches of 3-10 us of latency (in a
+// graph); at 4096 items and 12,600 pairs 34 against 58, with the gap closing by the
+// 2 us that another 1000 items or pairs cost one CTA, about where its arrays end.
+// ---------------------------------------------------------------------------
+constexpr int kSmThreads = 1024, kSmWarps = kSmThreads / 32;
+constexpr int kSmItems = 4096, kSmPairs = 24576, kSmTiles = 256;
+struct SmallSmem {
+    uint32_t key[2][kSmItems];  // depth bits; then each sorted item's first pair
+    uint16_t val[2][kSmItems];
+    uint32_t off[kSmItems];
+    uint32_t mask[kSmWarps][256];
+    uint16_t cnt[kSmWarps][256];
+    uint16_t p_item[kSmPairs];
+    uint8_t p_tile[kSmPairs], p_local[kSmPairs];  // tile; index in the item's rect
+    uint32_t len[kSmTiles];
+};
+
+// First place of each (warp, digit) in the sorted order from the counts in s.cnt; the
+// digit's total and start to thread d < 256. All threads.
+__device__ __forceinline__ void small_places(SmallSmem& s, uint32_t& tot, uint32_t& start) {
+    const int t = threadIdx.x;
+    tot = 0;
+    if (t < 256) {
+#pragma unroll 8
+        for (int q = 0; q < kSmWarps; q++) tot += s.cnt[q][t];
+    }
+    block_exclusive_scan<kSmThreads>(tot, start);
+    if (t < 256) {
+        uint32_t place = start;
+#pragma unroll 8
+        for (int q = 0; q < kSmWarps; q++) {
+            const uint32_t c = s.cnt[q][t];
+            s.cnt[q][t] = (uint16_t)place;
+            place += c;
+        }
+    }
+    __syncthreads();
+}
+
+// The place of a warp's key with digit d among its (warp, digit)'s keys, which have
+// s.cnt[w][d] before them: the lanes before it with the same digit, the count moved on.
+__device__ __forceinline__ uint32_t small_rank(SmallSmem& s, int w, unsigned d, bool valid) {
+    if (valid) atomicOr(&s.mask[w][d], 1u << (threadIdx.x & 31));
+    __syncwarp();
+    const uint32_t m = s.mask[w][d], before = s.cnt[w][d];
+    __syncwarp();
+    const unsigned lower = m & lanemask_lt();
+    if (valid && lower == 0) {
+        s.mask[w][d] = 0;
+        s.cnt[w][d] = (uint16_t)(before + __popc(m));
+    }
+    __syncwarp();
+    return before + __popc(lower);
+}
+
+__global__ void __launch_bounds__(kSmThreads, 1) k_sort_small(
+    const int32_t* __restrict__ n_tiles, const float4* __restrict__ rgb_depth, const ushort4* __restrict__ rect,
+    int64_t n, const __grid_constant__ gs_frame f, int n_items, int tiles, int64_t capacity, uint32_t* __restrict__ offset,
+    uint32_t* __restrict__ src, uint32_t* __restrict__ emit, uint32_t* __restrict__ range, uint32_t* __restrict__ order,
+    int64_t* __restrict__ count, int32_t* __restrict__ status) {
+    extern __shared__ __align__(16) uint8_t s_raw[];
+    SmallSmem& s = *reinterpret_cast<SmallSmem*>(s_raw);
+    const unsigned FULL = 0xffffffffu;
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    constexpr int kPer = kSmItems / kSmThreads;
+    for (int i = t; i < kSmWarps * 256; i += kSmThreads) {
+        (&s.mask[0][0])[i] = 0;
+        (&s.cnt[0][0])[i] = 0;
+    }
+    // 1. offsets in item order, visible items with their depths
+    uint32_t nv;
+    {
+        uint32_t nt[kPer], vis = 0, sum = 0, depth[kPer];
+#pragma unroll
+        for (int k = 0; k < kPer; k++) nt[k] = kPer * t + k < n_items ? (uint32_t)max(n_tiles[kPer * t + k], 0) : 0u;
+#pragma unroll
+        for (int k = 0; k < kPer; k++) {
+            depth[k] = nt[k] > 0 ? __float_as_uint(rgb_depth[kPer * t + k].w) : 0u;
+            vis += nt[k] > 0;
+            sum += nt[k];
+        }
+        uint32_t pos, slot;
+        nv = block_exclusive_scan<kSmThreads>(vis, pos);
+        block_exclusive_scan<kSmThreads>(sum, slot);
+#pragma unroll
+        for (int k = 0; k < kPer; k++) {
+            if (kPer * t + k >= n_items) break;
+            offset[kPer * t + k] = slot;
+            s.off[kPer * t + k] = slot;
+            slot += nt[k];
+            if (nt[k] > 0) {
+                s.key[0][pos] = depth[k];
+                s.val[0][pos++] = (uint16_t)(kPer * t + k);
+            }
+        }
+    }
+    __syncthreads();
+    // 2. stable sort by depth bits; a warp takes a contiguous span
+    int in = 0;
+    {
+        const int span = (int)((nv + kSmThreads - 1) / kSmThreads) * 32, b0 = w * span + lane;
+        for (int shift = 0; shift < 32; shift += 8) {
+            uint32_t kk[kPer], rank[kPer];
+#pragma unroll
+            for (int k = 0; k < kPer; k++) {
+                const bool valid = 32 * k < span && b0 + 32 * k < (int)nv;
+                kk[k] = valid ? s.key[in][b0 + 32 * k] : 0u;
+                rank[k] = small_rank(s, w, (kk[k] >> shift) & 255u, valid);
+            }
+            __syncthreads();
+            uint32_t tot, start;
+            small_places(s, tot, start);
+            const bool same = __syncthreads_or(t < 256 && nv > 0 && tot == nv);
+            if (!same) {
+#pragma unroll
+                for (int k = 0; k < kPer; k++)
+                    if (32 * k < span && b0 + 32 * k < (int)nv) {
+                        const uint32_t pos = s.cnt[w][(kk[k] >> shift) & 255u] + rank[k];
+                        s.key[in ^ 1][pos] = kk[k];
+                        s.val[in ^ 1][pos] = s.val[in][b0 + 32 * k];
+                    }
+                in ^= 1;
+            }
+            __syncthreads();
+            for (int i = t; i < kSmWarps * 256; i += kSmThreads) (&s.cnt[0][0])[i] = 0;
+            __syncthreads();
+        }
+    }
+    // 3. pairs in depth order: first pair of each sorted item, then a warp writes 32 items' pairs together
+    const uint32_t n32 = (uint32_t)n, magic = view_magic(n32);
+    uint32_t* first = s.key[in];
+    uint32_t total;
+    {
+        uint32_t c[kPer], sum = 0, pos;
+#pragma unroll
+        for (int k = 0; k < kPer; k++) {
+            c[k] = 0;
+            if (kPer * t + k < (int)nv) {
+                const uint32_t item = s.val[in][kPer * t + k];
+                c[k] = item_rect(rect[item], f, view_of(item, n32, magic)).cnt;
+            }
+            sum += c[k];
+        }
+        total = block_exclusive_scan<kSmThreads>(sum, pos);
+#pragma unroll
+        for (int k = 0; k < kPer; k++) {
+            if (kPer * t + k < (int)nv) first[kPer * t + k] = pos;
+            pos += c[k];
+        }
+    }
+    const uint32_t n_eff = (uint32_t)min((int64_t)total, capacity);
+    if (t == 0) {
+        *count = total;
+        *status = (int64_t)total > capacity ? GS_ERR_CAPACITY : GS_OK;
+    }
+    __syncthreads();
+    for (int g = w; g * 32 < (int)nv; g += kSmWarps) {
+        const int at = g * 32 + lane;
+        const bool have = at < (int)nv;
+        const uint32_t item = have ? s.val[in][at] : 0u;
+        const ItemRect q = item_rect(rect[item], f, view_of(item, n32, magic));
+        const uint32_t cnt = have ? q.cnt : 0u, start = have ? first[at] : 0xFFFFFFFFu;
+        const uint32_t t0 = q.base + q.y0 * q.tx + q.x0;
+        const uint32_t lo = __shfl_sync(FULL, start, 0);
+        const uint32_t hi = min(__reduce_max_sync(FULL, have ? start + cnt : 0u), n_eff);
+        for (uint32_t b = lo; b < hi; b += 32) {
+            const uint32_t j = b + lane;
+            int L = 0;  // the last item that starts at or before pair j (its pairs reach past j: empty items start later)
+#pragma unroll
+            for (int step = 16; step >= 1; step >>= 1) {
+                const uint32_t st = __shfl_sync(FULL, start, L + step);
+                if (L + step < 32 && st <= j) L += step;
+            }
+            const uint32_t st = __shfl_sync(FULL, start, L), it = __shfl_sync(FULL, item, L);
+            const uint32_t aw = __shfl_sync(FULL, q.wx, L), at0 = __shfl_sync(FULL, t0, L);
+            const uint32_t atx = __shfl_sync(FULL, q.tx, L);
+            if (j < hi) {
+                const uint32_t local = j - st, yy = local / aw;
+                s.p_item[j] = (uint16_t)it;
+                s.p_local[j] = (uint8_t)local;
+                s.p_tile[j] = (uint8_t)(at0 + yy * atx + (local - yy * aw));
+            }
+        }
+    }
+    __syncthreads();
+    // 4. stable counting sort by tile, written to the lists
+    const int span = (int)((n_eff + kSmThreads - 1) / kSmThreads) * 32, p0 = w * span, p1 = min(p0 + span, (int)n_eff);
+    for (int p = p0 + lane; p < p1; p += 32) atomicAdd(&s.mask[w][s.p_tile[p]], 1u);
+    __syncthreads();
+    for (int i = t; i < kSmWarps * 256; i += kSmThreads) {
+        (&s.cnt[0][0])[i] = (uint16_t)(&s.mask[0][0])[i];
+        (&s.mask[0][0])[i] = 0;
+    }
+    __syncthreads();
+    uint32_t tot, start;
+    small_places(s, tot, start);
+    if (t < tiles) {
+        range[2 * t] = tot ? start : 0u;
+        range[2 * t + 1] = tot ? start + tot : 0u;
+        s.len[t] = min(tot, 0xFFFFu);
+    }
+    for (int p = p0; p < p1; p += 32) {
+        const bool valid = p + lane < p1;
+        const uint32_t item = valid ? s.p_item[p + lane] : 0u, local = valid ? s.p_local[p + lane] : 0u;
+        const uint32_t dest = small_rank(s, w, valid ? s.p_tile[p + lane] : 0u, valid);
+        if (valid) {
+            src[dest] = item;
+            emit[dest] = s.off[item] + local;
+        }
+    }
+    // 5. work order: tiles by decreasing pair count
+    if (order) {
+        __syncthreads();
+        if (t < tiles) {
+            uint32_t r = 0;
+            for (int u = 0; u < tiles; u++) r += s.len[u] > s.len[t] || (s.len[u] == s.len[t] && u < t);
+            order[r] = (uint32_t)t;
+        }
+    }
+}
+
+// The rule: what the CTA's arrays hold (a rect has at most its view's tiles).
+static bool small_fits(int64_t n, int64_t n_items, int64_t n_tiles, int64_t capacity) {
+    const int64_t most = n * n_tiles < capacity ? n * n_tiles : capacity;
+    return n_items <= kSmItems && n_tiles <= kSmTiles && most <= kSmPairs;
+}
+
 struct SortWs {
     uint32_t *vk0, *vv0, *vk1, *vv1, *group_off, *first_group, *pk0, *pk1, *misc;
     uint2 *psrc, *psrc2;
@@ -1302,6 +1534,19 @@ extern "C" int gs_sort(const gs_projected* p, int64_t n, const gs_frame* f, cons
     uint32_t* n_vis = w.misc;        // visible item count
     uint32_t* n_eff = w.misc + 2;    // pairs actually stored
     int32_t* err = (int32_t*)(w.misc + 3);  // GS_ERR_TIMEOUT from a look-back wait
+    if (n_items > 0 && small_fits(n, n_items, n_tiles_total, out->capacity)) {
+        if (cudaFuncSetAttribute(k_sort_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmallSmem)) !=
+            cudaSuccess) {
+            (void)cudaGetLastError();
+            return GS_ERR_CUDA;
+        }
+        k_sort_small<<<1, kSmThreads, sizeof(SmallSmem), s>>>(
+            p->n_tiles, (const float4*)p->rgb_depth, (const ushort4*)p->rect, n, *f, (int)n_items, (int)n_tiles_total,
+            out->capacity, out->offset, out->src, out->emit, out->range, out->order, out->count, out->status);
+        count_launch();
+        GS_CUDA_CHECK_LAUNCH();
+        return GS_OK;
+    }
     cudaMemsetAsync(out->range, 0, sizeof(uint32_t) * 2 * n_tiles_total, s);
     if (n_items == 0) {
         k_no_pairs<<<1, 1, 0, s>>>(out->count, out->status);
