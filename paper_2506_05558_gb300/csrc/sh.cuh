@@ -18,14 +18,14 @@ constexpr float kSH3c = 0.4570457994644658f;   // sqrt(21/(2 pi))/4
 constexpr float kSH3d = 0.3731763325901154f;   // sqrt(7/pi)/4
 constexpr float kSH3e = 1.445305721320277f;    // sqrt(105/pi)/4
 
-__device__ __forceinline__ void sh_eval_basis(int deg, float x, float y, float z, float* Y) {
+// The basis from the direction and its squares.
+__device__ __forceinline__ void sh_eval_basis(int deg, float x, float y, float z, float xx, float yy, float zz, float* Y) {
     Y[0] = kSH0;
     if (deg < 1) return;
     Y[1] = -kSH1 * y;
     Y[2] = kSH1 * z;
     Y[3] = -kSH1 * x;
     if (deg < 2) return;
-    const float xx = x * x, yy = y * y, zz = z * z;
     Y[4] = kSH2a * x * y;
     Y[5] = -kSH2a * y * z;
     Y[6] = kSH2b * (2.f * zz - xx - yy);
@@ -39,6 +39,9 @@ __device__ __forceinline__ void sh_eval_basis(int deg, float x, float y, float z
     Y[13] = -kSH3c * x * (4.f * zz - xx - yy);
     Y[14] = kSH3e * z * (xx - yy);
     Y[15] = -kSH3a * x * (xx - 3.f * yy);
+}
+__device__ __forceinline__ void sh_eval_basis(int deg, float x, float y, float z, float* Y) {
+    sh_eval_basis(deg, x, y, z, x * x, y * y, z * z, Y);
 }
 
 // Gradient of f = sum_k w_k Y_k with respect to the direction components
