@@ -12,7 +12,9 @@
 // are formed once after the last view, and for SH degree d the 3 (d + 1)^2
 // coefficient gradients gc_v[ch] Y_v[k] (summed after the view loop from
 // shared memory for up to 16 views) - so each gradient row is written once,
-// without atomics. Each view's pose gradient is summed over the warp's 32
+// without atomics. SH rows pass through shared memory both ways, a warp's 32 as whole
+// runs (1M Gaussians, eight 1080p views: 334 us, 387 with each thread at its own
+// 192-byte row; issue and L1 share the rest). Each view's pose gradient is summed over the warp's 32
 // Gaussians by a fixed xor tree and over the CTA's four warps in order into
 // one partial per (view, CTA), and those are summed by k_pose_reduce in a
 // fixed order: the whole backward pass
@@ -23,6 +25,7 @@
 
 namespace gs {
 
+constexpr int kPBPitch = 13;  // float4 from Gaussian to Gaussian in shared memory: no bank conflicts
 constexpr int kPBThreads = 128;  // threads (Gaussians) per CTA of k_project_bwd, one pose partial per view
 
 // Record of item i: (du dv dA dB | dC dop dr dg | db 0 0 0), written only for
@@ -108,8 +111,12 @@ __global__ void __launch_bounds__(kPBThreads, DV > 0 ? 4 : 1) k_project_bwd(
     constexpr int NC = (SHD + 1) * (SHD + 1);  // SH coefficients per channel
     constexpr int NR = (3 * NC + 3) / 4;       // float4 rows of SH coefficients in use
     constexpr int NWP = kPBThreads / 32;
-    __shared__ gs_camera s_cam[GS_MAX_VIEWS];
-    __shared__ float s_pose[GS_MAX_VIEWS][NWP][6];  // each warp's pose partial per view
+    constexpr int NV = DV > 0 ? DV : GS_MAX_VIEWS;
+    __shared__ gs_camera s_cam[NV];
+    __shared__ float s_pose[NV][NWP][6];  // each warp's pose partial per view
+    // SH rows of the CTA's Gaussians: the coefficients, then their gradients (a thread's own row is
+    // 192 bytes from the next one's: read or written directly, a warp's access touches 32 lines)
+    __shared__ __align__(16) float4 s_sh[kPBThreads * kPBPitch];
     const unsigned FULL = 0xffffffffu;
     const int nv = f.n_views;
     for (int i = threadIdx.x; i < nv * (int)(sizeof(gs_camera) / 4); i += kPBThreads)
@@ -144,7 +151,9 @@ __global__ void __launch_bounds__(kPBThreads, DV > 0 ? 4 : 1) k_project_bwd(
     for (int k = 0; k < 9; k++) RS[k] *= sv[k % 3];
     const float opa = 1.f / (1.f + expf(-mo.w));
     float a3 = 0.f;  // sum over views of dL/d(opacity) x the 2-D filter factor
-    const float4* shg = sh + 12 * g;
+    float4* rows = s_sh + (threadIdx.x - lane) * kPBPitch;  // the warp's
+    const float4* shg = rows + lane * kPBPitch;
+    bool have = false;
     // per-Gaussian sums over the views (in view order)
     // and H = sum_v R_v^T dL/dT_v (T_v = R_v Rq diag(s')): the scale and rotation gradients are
     // linear in H and are formed once, after the view loop
@@ -176,6 +185,23 @@ __global__ void __launch_bounds__(kPBThreads, DV > 0 ? 4 : 1) k_project_bwd(
             r0_nx = rec[3 * nx];
             r1_nx = rec[3 * nx + 1];
             r2_nx = rec[3 * nx + 2];
+        }
+        // the SH rows of the warp's Gaussians that a view lists for the first time
+        const unsigned need = __ballot_sync(FULL, nt > 0 && !have);
+        if (need) {
+            const float4* first = sh + 12 * (g - lane);
+#pragma unroll
+            for (int k = 0; k < NR; k++) {
+                const int gl = (32 * k + lane) / NR, r = (32 * k + lane) % NR;
+                if ((need >> gl) & 1u)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                                     (uint32_t)__cvta_generic_to_shared(rows + gl * kPBPitch + r)),
+                                 "l"(first + 12 * gl + r)
+                                 : "memory");
+            }
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            __syncwarp();
+            have |= nt > 0;
         }
         float pose[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
         if (nt > 0) {
@@ -369,13 +395,12 @@ __global__ void __launch_bounds__(kPBThreads, DV > 0 ? 4 : 1) k_project_bwd(
         for (int q = 0; q < NWP; q++) pv += s_pose[v][q][c];
         pose_part[((int64_t)v * gridDim.x + blockIdx.x) * 6 + c] = pv;
     }
-    if (!valid) return;
     if constexpr (DV > 0) {
         // the SH-coefficient gradients, summed over the views in order as above
 #pragma unroll
         for (int c = 0; c < 3 * NC; c++) ash[c] = 0.f;
         const int t = threadIdx.x;
-        const float4 me = mean_opa[g];
+        const float4 me = valid ? mean_opa[g] : zero4;
         for (int v = 0; v < nv; v++) {
             if (!((vmask >> v) & 1u)) continue;
             const float gc[3] = {s_gd[v][0][t], s_gd[v][1][t], s_gd[v][2][t]};
@@ -433,27 +458,39 @@ __global__ void __launch_bounds__(kPBThreads, DV > 0 ? 4 : 1) k_project_bwd(
         const float qd = gq[0] * qw + gq[1] * qx + gq[2] * qy + gq[3] * qz;
         oq = make_float4((gq[0] - qw * qd) * qi, (gq[1] - qx * qd) * qi, (gq[2] - qy * qd) * qi, (gq[3] - qz * qd) * qi);
     }
-    if (cfg.accumulate) {
-        const float4 a = g_mean_opa[g], b = g_scale[g], q = g_quat[g];
-        om.x += a.x; om.y += a.y; om.z += a.z; om.w += a.w;
-        os.x += b.x; os.y += b.y; os.z += b.z; os.w += b.w;
-        oq.x += q.x; oq.y += q.y; oq.z += q.z; oq.w += q.w;
-    }
-    g_mean_opa[g] = om;
-    g_scale[g] = os;
-    g_quat[g] = oq;
-#pragma unroll
-    for (int r = 0; r < 12; r++) {
-        float4 val = make_float4(4 * r < 3 * NC ? ash[4 * r] : 0.f, 4 * r + 1 < 3 * NC ? ash[4 * r + 1] : 0.f,
-                                 4 * r + 2 < 3 * NC ? ash[4 * r + 2] : 0.f, 4 * r + 3 < 3 * NC ? ash[4 * r + 3] : 0.f);
+    if (valid) {
         if (cfg.accumulate) {
-            const float4 old = g_sh[12 * g + r];
+            const float4 a = g_mean_opa[g], b = g_scale[g], q = g_quat[g];
+            om.x += a.x; om.y += a.y; om.z += a.z; om.w += a.w;
+            os.x += b.x; os.y += b.y; os.z += b.z; os.w += b.w;
+            oq.x += q.x; oq.y += q.y; oq.z += q.z; oq.w += q.w;
+        }
+        g_mean_opa[g] = om;
+        g_scale[g] = os;
+        g_quat[g] = oq;
+        uint8_t* vd = visible + g;
+        *vd = (vis || (cfg.accumulate && *vd)) ? 1 : 0;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < NR; r++)
+        rows[lane * kPBPitch + r] =
+            make_float4(4 * r < 3 * NC ? ash[4 * r] : 0.f, 4 * r + 1 < 3 * NC ? ash[4 * r + 1] : 0.f,
+                        4 * r + 2 < 3 * NC ? ash[4 * r + 2] : 0.f, 4 * r + 3 < 3 * NC ? ash[4 * r + 3] : 0.f);
+    __syncwarp();
+    const int64_t g0 = g - lane;
+    float4* out = g_sh + 12 * g0;
+#pragma unroll
+    for (int k = 0; k < 12; k++) {
+        const int i = 32 * k + lane, gl = i / 12, r = i % 12;
+        if (g0 + gl >= n) break;
+        float4 val = r < NR ? rows[gl * kPBPitch + r] : zero4;
+        if (cfg.accumulate) {
+            const float4 old = out[i];
             val.x += old.x; val.y += old.y; val.z += old.z; val.w += old.w;
         }
-        g_sh[12 * g + r] = val;
+        out[i] = val;
     }
-    uint8_t* vd = visible + g;
-    *vd = (vis || (cfg.accumulate && *vd)) ? 1 : 0;
 }
 
 // dL/dxi of view v = sum over CTAs of pose_part[v][b][6], fixed tree order.
