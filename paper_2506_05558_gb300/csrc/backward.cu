@@ -31,59 +31,106 @@ constexpr int kPBThreads = 128;  // threads (Gaussians) per CTA of k_project_bwd
 // Record of item i: (du dv dA dB | dC dop dr dg | db 0 0 0), written only for
 // items with pairs (zeros after a pair-buffer overflow); also the 9 values to
 // d_proj (when given).
-// The runs of a warp's 32 consecutive items form one contiguous slot range:
-// the warp loads it window by window into shared memory with coalesced loads,
-// then each lane adds the slots of its own run in slot order.
-constexpr int kGatherWin = 128;  // slots per window and warp
+// The runs of a warp's 32 consecutive items form one contiguous slot range: the warp
+// copies it window by window into shared memory (asynchronously, the next
+// window or the next 32 items' first one while this one is added), then each lane adds
+// the slots of its own run in slot order. A warp takes kGatherRuns x 32 items, whose
+// counts and offsets it loads at once. 8M items, 15.8M pairs: 218 us for 910 MB
+// (283 with one run per warp and loads through registers).
+constexpr int kGatherWin = 80;  // slots per window and warp
 constexpr int kGatherWarps = 8;
+constexpr int kGatherSmem = 2 * kGatherWarps * kGatherWin * 36;
 
+template <int kGatherRuns>
 __global__ void __launch_bounds__(32 * kGatherWarps) k_item_partials(
     int64_t n_items, const int32_t* __restrict__ n_tiles, const uint32_t* __restrict__ offset,
     const float4* __restrict__ part0, const float4* __restrict__ part1, const float* __restrict__ part2,
     int64_t capacity, const int32_t* __restrict__ sort_status, float4* __restrict__ rec, float* __restrict__ d_proj) {
-    __shared__ float4 s0[kGatherWarps][kGatherWin];
-    __shared__ float4 s1[kGatherWarps][kGatherWin];
-    __shared__ float s2[kGatherWarps][kGatherWin];
+    extern __shared__ __align__(16) uint8_t s_raw[];
+    struct Win {
+        float4 a[kGatherWin], b[kGatherWin];
+        float c[kGatherWin];
+    };
+    static_assert(sizeof(Win) % 16 == 0);
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t item = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool in = item < n_items;
-    int nt = in ? n_tiles[item] : 0;
-    const uint32_t off = in ? offset[item] : 0u;
+    Win* win = reinterpret_cast<Win*>(s_raw) + 2 * w;
+    const int64_t first = ((int64_t)blockIdx.x * kGatherWarps + w) * (32 * kGatherRuns);
+    if (first >= n_items) return;  // no CTA-wide synchronisation below
     const bool ok = *sort_status == GS_OK;  // after an overflow some slots were never written: no gradient
-    // slots past the pair buffer's capacity were never written (overflowed sort)
-    const int64_t run = (ok && nt > 0) ? max((int64_t)0, min((int64_t)nt, capacity - (int64_t)off)) : 0;
-    const int64_t beg = off, end = off + run;
-    const int64_t lo = __reduce_min_sync(FULL, run > 0 ? (unsigned)beg : 0xffffffffu);
-    const int64_t hi = __reduce_max_sync(FULL, run > 0 ? (unsigned)end : 0u);
-    float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0;
-    float a2 = 0.f;
-    for (int64_t base = lo; base < hi; base += kGatherWin) {
-        const int cnt = (int)min((int64_t)kGatherWin, hi - base);
-        for (int j = lane; j < cnt; j += 32) {
-            s0[w][j] = part0[base + j];
-            s1[w][j] = part1[base + j];
-            s2[w][j] = part2[base + j];
-        }
-        __syncwarp();
-        const int64_t from = max(beg, base), to = min(end, base + cnt);
-        for (int64_t q = from; q < to; q++) {
-            const float4 p0 = s0[w][q - base], p1 = s1[w][q - base];
-            a0.x += p0.x; a0.y += p0.y; a0.z += p0.z; a0.w += p0.w;
-            a1.x += p1.x; a1.y += p1.y; a1.z += p1.z; a1.w += p1.w;
-            a2 += s2[w][q - base];
-        }
-        __syncwarp();
+    int nt[kGatherRuns];
+    uint32_t off[kGatherRuns], lo[kGatherRuns], hi[kGatherRuns];  // of the lane; of the run's slots
+#pragma unroll
+    for (int k = 0; k < kGatherRuns; k++) {
+        const int64_t item = first + 32 * k + lane;
+        nt[k] = item < n_items ? n_tiles[item] : 0;
+        off[k] = item < n_items ? offset[item] : 0u;
     }
-    if (!in || nt <= 0) return;  // an item without pairs has no record (its reader skips it)
-    rec[3 * item] = a0;
-    rec[3 * item + 1] = a1;
-    rec[3 * item + 2] = make_float4(a2, 0.f, 0.f, 0.f);
-    if (d_proj && nt > 0) {
-        float* o = d_proj + 9 * item;
-        o[0] = a0.x; o[1] = a0.y; o[2] = a0.z; o[3] = a0.w; o[4] = a1.x; o[5] = a1.y; o[6] = a1.z; o[7] = a1.w;
-        o[8] = a2;
+#pragma unroll
+    for (int k = 0; k < kGatherRuns; k++) {
+        // slots past the pair buffer's capacity were never written (overflowed sort)
+        const int64_t run = (ok && nt[k] > 0) ? max((int64_t)0, min((int64_t)nt[k], capacity - (int64_t)off[k])) : 0;
+        lo[k] = __reduce_min_sync(FULL, run > 0 ? off[k] : 0xffffffffu);
+        hi[k] = __reduce_max_sync(FULL, run > 0 ? (uint32_t)(off[k] + run) : 0u);
     }
+    auto fetch = [&](uint32_t base, uint32_t end, Win& to) {
+        const uint32_t cnt = base < end ? min(end - base, (uint32_t)kGatherWin) : 0u;
+        for (uint32_t j = lane; j < cnt; j += 32) {
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(&to.a[j])),
+                         "l"(part0 + base + j)
+                         : "memory");
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(&to.b[j])),
+                         "l"(part1 + base + j)
+                         : "memory");
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(&to.c[j])),
+                         "l"(part2 + base + j)
+                         : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    fetch(lo[0], hi[0], win[0]);
+    int buf = 0;
+#pragma unroll
+    for (int k = 0; k < kGatherRuns; k++) {
+        const uint32_t beg = off[k];
+        const uint32_t end = ok && nt[k] > 0 ? (uint32_t)min((int64_t)beg + nt[k], max(capacity, (int64_t)beg)) : beg;
+        float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0;
+        float a2 = 0.f;
+        uint32_t base = lo[k];
+        for (;;) {
+            const bool more = base < hi[k] && hi[k] - base > kGatherWin;  // another window of this run
+            if (more) fetch(base + kGatherWin, hi[k], win[buf ^ 1]);
+            else if (k + 1 < kGatherRuns) fetch(lo[k + 1 < kGatherRuns ? k + 1 : k], hi[k + 1 < kGatherRuns ? k + 1 : k], win[buf ^ 1]);
+            else asm volatile("cp.async.commit_group;" ::: "memory");
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+            __syncwarp();
+            const Win& s = win[buf];
+            if (base < hi[k]) {
+                const uint32_t to = min(end, hi[k] - base > kGatherWin ? base + kGatherWin : hi[k]);
+                for (uint32_t q = max(beg, base); q < to; q++) {
+                    const float4 p0 = s.a[q - base], p1 = s.b[q - base];
+                    a0.x += p0.x; a0.y += p0.y; a0.z += p0.z; a0.w += p0.w;
+                    a1.x += p1.x; a1.y += p1.y; a1.z += p1.z; a1.w += p1.w;
+                    a2 += s.c[q - base];
+                }
+            }
+            __syncwarp();
+            buf ^= 1;
+            if (!more) break;
+            base += kGatherWin;
+        }
+        const int64_t item = first + 32 * k + lane;
+        if (item >= n_items || nt[k] <= 0) continue;  // an item without pairs has no record (its reader skips it)
+        rec[3 * item] = a0;
+        rec[3 * item + 1] = a1;
+        rec[3 * item + 2] = make_float4(a2, 0.f, 0.f, 0.f);
+        if (d_proj) {
+            float* o = d_proj + 9 * item;
+            o[0] = a0.x; o[1] = a0.y; o[2] = a0.z; o[3] = a0.w; o[4] = a1.x; o[5] = a1.y; o[6] = a1.z; o[7] = a1.w;
+            o[8] = a2;
+        }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
 // Rotation matrix (row-major) of the unit quaternion (w, x, y, z).
@@ -587,8 +634,15 @@ extern "C" int gs_project_bwd(const gs_gaussians* g, const gs_camera* cams, cons
     }
     const int64_t nb = ceil_div(g->n, kPBThreads);  // CTAs of k_project_bwd (pose partials per view)
     const int64_t n_items = (int64_t)f->n_views * g->n;
-    k_item_partials<<<(unsigned)ceil_div(n_items, 32 * kGatherWarps), 32 * kGatherWarps, 0, s>>>(
-        n_items, p->n_tiles, pairs->offset, w.part0, w.part1, w.part2, pairs->capacity, pairs->status, w.rec, d_proj);
+    // four runs per warp once that fills the 608 CTAs that are resident; below, latency
+    // counts (1000 items: 30 us of adjoint against 32)
+    constexpr int kGatherItems = 32 * kGatherWarps;
+#define GS_GATHER(RUNS)                                                                                          \
+    k_item_partials<RUNS><<<(unsigned)ceil_div(n_items, RUNS * kGatherItems), kGatherItems, kGatherSmem, s>>>(   \
+        n_items, p->n_tiles, pairs->offset, w.part0, w.part1, w.part2, pairs->capacity, pairs->status, w.rec, d_proj)
+    if (n_items >= 4 * kGatherItems * 608) GS_GATHER(4);
+    else GS_GATHER(1);
+#undef GS_GATHER
     count_launch();
     const unsigned grid = (unsigned)ceil_div(g->n, kPBThreads);
 #define GS_PB(D)                                                                                                \
