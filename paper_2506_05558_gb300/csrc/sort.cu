@@ -10,9 +10,9 @@
 // decoupled look-back), the digits counted by the kernel that writes the keys; the
 // tile sort carries every pair's (item, emission slot) and its last pass writes
 // them to the output lists. 8 views of 1080p, 1M Gaussians (5.8M visible items, 15.8M
-// pairs): 719 us, of which the passes over items take 188 and those over pairs 230
-// (1049, 274 and 333 with separate scans, histograms, and values gathered from global
-// memory in sorted order). Element counts are read from device memory, so the
+// pairs): 659 us in a graph, of which the passes over items take 188 and those over
+// pairs 230 (970, 274 and 333 with separate scans, histograms, and values gathered from
+// global memory in sorted order). Element counts are read from device memory, so the
 // whole sort is enqueued without a host sync and can be captured in a CUDA
 // graph. The reduce-then-scan scan and radix sort below serve the library's
 // other compactions and sorts (spawning, anchors).
@@ -632,9 +632,18 @@ __device__ __forceinline__ void add_digit_counts(const uint32_t (*s_h)[256], int
     }
 }
 
-// Digit counts of given keys, and the first pass's look-back words zeroed.
+// Keys per CTA of a pass over at most n_max keys: 16 rounds of 32 per warp, or 8 where
+// even those tiles are about one round of the resident CTAs (three per SM), and a
+// pass takes as long as one tile does (the sort of 150K items and 410K pairs: 86 us
+// against 96; of 1M and 2M, where only the items' passes take it: 148 against 150).
+constexpr int64_t kFewKeys = 1 << 20;
+static int onesweep_tile(int64_t n_max) { return n_max <= kFewKeys ? kRadixTile / 2 : kRadixTile; }
+static int64_t onesweep_blocks(int64_t n_max) { return ceil_div(n_max, onesweep_tile(n_max)); }
+
+// Digit counts of given keys, and the first pass's look-back words zeroed; a CTA counts
+// two of the passes' smaller tiles.
 __global__ void __launch_bounds__(256) k_onesweep_hist(const uint32_t* __restrict__ keys, int64_t n, int passes,
-                                                       SortCtl* ctl, LbWords words) {
+                                                       SortCtl* ctl, LbWords words, int64_t blocks) {
     __shared__ uint32_t s_h[kMaxPasses][256];
     for (int i = threadIdx.x; i < kMaxPasses * 256; i += 256) (&s_h[0][0])[i] = 0;
     __syncthreads();
@@ -649,7 +658,7 @@ __global__ void __launch_bounds__(256) k_onesweep_hist(const uint32_t* __restric
     for (int it = 0; it < kRadixIters; it++)
         if (t0 + it * 256 + threadIdx.x < n)
             for (int p = 0; p < passes; p++) atomicAdd(&s_h[p][(k[it] >> (8 * p)) & 255u], 1u);
-    lb_zero(words, blockIdx.x);
+    for (int64_t b = blockIdx.x; b < blocks; b += gridDim.x) lb_zero(words, b);
     add_digit_counts(s_h, passes, ctl, gridDim.x);
 }
 
@@ -670,20 +679,21 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_al
 // by an OR of lane bits per digit: 13 instructions a round, 50 by nine ballots, and
 // match.any was slower than both), and the sorted order fetches them from shared
 // memory. 5.8M items: 45 us a pass (70 before), 15.8M pairs: 115 (166).
-template <class V>
+template <class V, int ITERS>
 __global__ void __launch_bounds__(kRadixThreads, 3) k_onesweep_pass(
     const uint32_t* __restrict__ kin, const V* __restrict__ vin, uint32_t* __restrict__ kout, V* __restrict__ vout,
     uint32_t* __restrict__ out_x, uint32_t* __restrict__ out_y, int64_t n_max, const uint32_t* n_dev, int pass,
     SortCtl* ctl, LbWords words, LbWords next, int32_t* err) {
+    constexpr int kTile = kRadixThreads * ITERS, kSpan = 32 * ITERS;  // keys per CTA and per warp
     __shared__ uint16_t cnt[kRadixWarps][256];  // keys so far per warp and digit, then the warp's first place in the tile
     __shared__ uint32_t goff[256];              // global minus tile-local start of each digit
-    __shared__ uint32_t s_k[kRadixTile];        // the sorted tile's keys
-    __shared__ uint16_t s_i[kRadixTile];        // and their places in the input
-    __shared__ __align__(16) V s_v[kRadixTile];  // the input's values
+    __shared__ uint32_t s_k[kTile];        // the sorted tile's keys
+    __shared__ uint16_t s_i[kTile];        // and their places in the input
+    __shared__ __align__(16) V s_v[kTile];  // the input's values
     __shared__ uint32_t s_tile;
     // while ranking: lanes whose key of this round has the digit, per warp
     uint32_t(*mask)[256] = reinterpret_cast<uint32_t(*)[256]>(s_k);
-    static_assert(kRadixTile >= kRadixWarps * 256);
+    static_assert(kTile >= kRadixWarps * 256);
     const int shift = 8 * pass;
     if (threadIdx.x == 0) s_tile = atomicAdd(&ctl->ticket[pass], 1u);
     for (int i = threadIdx.x; i < kRadixWarps * 256; i += kRadixThreads) {
@@ -694,23 +704,23 @@ __global__ void __launch_bounds__(kRadixThreads, 3) k_onesweep_pass(
     const int64_t tile = s_tile;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t n = valid_count(n_max, n_dev);
-    const int64_t b0 = tile * kRadixTile;
+    const int64_t b0 = tile * kTile;
     if (b0 >= n) return;  // uniform over the CTA
     if (next.tile) lb_zero(next, tile);
-    const int64_t base = b0 + (int64_t)w * kRadixWarpSpan;
-    const int rem = (int)min(n - base, (int64_t)kRadixWarpSpan) - lane;
+    const int64_t base = b0 + (int64_t)w * kSpan;
+    const int rem = (int)min(n - base, (int64_t)kSpan) - lane;
     const uint32_t* kp = kin + base + lane;
-    const int cnt_block = (int)min((int64_t)kRadixTile, n - b0);
+    const int cnt_block = (int)min((int64_t)kTile, n - b0);
     // the values travel to shared memory while the keys are ranked
     constexpr int kPer = 16 / (int)sizeof(V);
 #pragma unroll
-    for (int i = threadIdx.x * kPer; i < kRadixTile; i += kRadixThreads * kPer)
+    for (int i = threadIdx.x * kPer; i < kTile; i += kRadixThreads * kPer)
         if (i < cnt_block) cp_async16(s_v + i, vin + b0 + i, min((cnt_block - i) * (int)sizeof(V), 16));
-    uint32_t kk[kRadixIters], rank[kRadixIters];
+    uint32_t kk[ITERS], rank[ITERS];
 #pragma unroll
-    for (int it = 0; it < kRadixIters; it++) kk[it] = 32 * it < rem ? load_now(kp + 32 * it) : 0u;
+    for (int it = 0; it < ITERS; it++) kk[it] = 32 * it < rem ? load_now(kp + 32 * it) : 0u;
 #pragma unroll
-    for (int it = 0; it < kRadixIters; it++) {
+    for (int it = 0; it < ITERS; it++) {
         const bool valid = 32 * it < rem;
         const unsigned d = (kk[it] >> shift) & 255u;
         if (valid) atomicOr(&mask[w][d], 1u << lane);
@@ -741,11 +751,11 @@ __global__ void __launch_bounds__(kRadixThreads, 3) k_onesweep_pass(
     }
     __syncthreads();
 #pragma unroll
-    for (int it = 0; it < kRadixIters; it++) {
+    for (int it = 0; it < ITERS; it++) {
         if (32 * it < rem) {
             const uint32_t pos = cnt[w][(kk[it] >> shift) & 255u] + rank[it];
             s_k[pos] = kk[it];
-            s_i[pos] = (uint16_t)(w * kRadixWarpSpan + lane + 32 * it);
+            s_i[pos] = (uint16_t)(w * kSpan + lane + 32 * it);
         }
     }
     goff[threadIdx.x] = ctl->count[pass][threadIdx.x] + look_back(words, tile, tot, err) - ex;
@@ -772,7 +782,7 @@ __global__ void __launch_bounds__(kRadixThreads, 3) k_onesweep_pass(
 
 // Look-back words of one radix pass over at most n_max keys.
 static int64_t onesweep_words(int64_t n_max) {
-    const int64_t tiles = radix_blocks(n_max);
+    const int64_t tiles = onesweep_blocks(n_max);
     return 256 * (tiles + 2 * lb_groups(tiles));
 }
 
@@ -787,14 +797,16 @@ template <class V>
 static bool onesweep_passes(uint32_t* ka, V* va, uint32_t* kb, V* vb, int64_t n_max, const uint32_t* n_dev, int bits,
                             SortCtl* ctl, uint64_t* wa, uint64_t* wb, int32_t* err, cudaStream_t s,
                             uint32_t* out_x = nullptr, uint32_t* out_y = nullptr) {
-    const int64_t nb = radix_blocks(n_max);
+    const int64_t nb = onesweep_blocks(n_max);
+    const auto kernel = onesweep_tile(n_max) == kRadixTile ? k_onesweep_pass<V, kRadixIters>
+                                                           : k_onesweep_pass<V, kRadixIters / 2>;
     const int passes = (bits + 7) / 8;
     bool in_b = false;
     for (int p = 0; p < passes; p++) {
         const bool last = p + 1 == passes;
         const LbWords w = lb_words((p & 1) ? wb : wa, nb);
         const LbWords wn = last ? LbWords{} : lb_words((p & 1) ? wa : wb, nb);
-        k_onesweep_pass<V><<<(unsigned)nb, kRadixThreads, 0, s>>>(
+        kernel<<<(unsigned)nb, kRadixThreads, 0, s>>>(
             in_b ? kb : ka, in_b ? vb : va, in_b ? ka : kb, in_b ? va : vb, last ? out_x : nullptr,
             last ? out_y : nullptr, n_max, n_dev, p, ctl, w, wn, err);
         count_launch();
@@ -1092,7 +1104,7 @@ __global__ void __launch_bounds__(kDupThreads, 5) k_duplicate(
     const uint32_t* __restrict__ sorted_item, const uint32_t* n_vis, const ushort4* __restrict__ rect, int64_t n,
     const __grid_constant__ gs_frame f, const uint32_t* n_eff, const uint32_t* __restrict__ group_off,
     const uint32_t* __restrict__ first_group, const uint32_t* __restrict__ offset, uint32_t* __restrict__ pkey,
-    uint2* __restrict__ psrc, int passes, SortCtl* sort, LbWords sort_words) {
+    uint2* __restrict__ psrc, int passes, SortCtl* sort, LbWords sort_words, int sort_tile) {
     const unsigned FULL = 0xffffffffu;
     __shared__ uint32_t s_h[kMaxPasses][256];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1103,7 +1115,7 @@ __global__ void __launch_bounds__(kDupThreads, 5) k_duplicate(
     const int64_t spans = (n_pairs + kDupPairs - 1) / kDupPairs;
     const int64_t span = (spans + gridDim.x - 1) / gridDim.x * kDupPairs;
     const int64_t p0 = blockIdx.x * span, p1 = min(p0 + span, n_pairs);
-    for (int64_t t = (p0 + kRadixTile - 1) / kRadixTile; t * kRadixTile < p1; t++) lb_zero(sort_words, t);
+    for (int64_t t = (p0 + sort_tile - 1) / sort_tile; t * sort_tile < p1; t++) lb_zero(sort_words, t);
     if (p0 < p1) {
         // the loads of a warp's next two groups are in flight while it writes one
         int64_t g = first_group[p0 / kDupPairs] + warp;
@@ -1461,18 +1473,18 @@ struct SortWs {
     uint64_t *wa, *wb;     // radix look-back words (zeroed by the kernels)
 };
 
-// One chunk per CTA, all of them resident; at least 256 items each.
+// One chunk per CTA, all of them resident, at least 1024 items each. Fewer CTAs look back
+// over fewer words, more of them gather faster: 152K, 750K and 5.8M visible items
+// took 5 and 6 us less and 4 us more of a sort with at most 304 than with 608.
 static int64_t dup_ctas(int64_t n_items) {
-    const int64_t g = ceil_div(n_items, 256);
-    return g < scan_ctas() ? g : scan_ctas();
+    const int64_t g = ceil_div(n_items, 1024), most = n_items < ((int64_t)4 << 20) ? scan_ctas() / 2 : scan_ctas();
+    return g < most ? g : most;
 }
 
 static SortWs carve_sort(char* base, size_t cap_bytes, int64_t n_items, int64_t capacity, int64_t n_tiles,
                          size_t* used) {
     Carve c{base, 0, cap_bytes};
     SortWs w;
-    int64_t m = n_items > capacity ? n_items : capacity;
-    m = m > n_tiles ? m : n_tiles;
     const size_t z0 = c.used;
     w.misc = c.take<uint32_t>(8);
     w.scan_ctl = c.take<ScanCtl>(2);
@@ -1493,8 +1505,11 @@ static SortWs carve_sort(char* base, size_t cap_bytes, int64_t n_items, int64_t 
     w.tv0 = c.take<uint32_t>(n_tiles);
     w.tk1 = c.take<uint32_t>(n_tiles);
     w.tv1 = c.take<uint32_t>(n_tiles);
-    w.wa = c.take<uint64_t>(onesweep_words(m));
-    w.wb = c.take<uint64_t>(onesweep_words(m));
+    int64_t words = onesweep_words(n_items);  // the most that one of the three sorts needs
+    for (const int64_t k : {capacity, n_tiles})
+        if (onesweep_words(k) > words) words = onesweep_words(k);
+    w.wa = c.take<uint64_t>(words);
+    w.wb = c.take<uint64_t>(words);
     *used = c.used;
     return w;
 }
@@ -1557,9 +1572,10 @@ extern "C" int gs_sort(const gs_projected* p, int64_t n, const gs_frame* f, cons
     cudaMemsetAsync(w.misc, 0, w.zero_bytes, s);
     // 1. emission slots, and the visible items (in item order) with their depth keys
     const int64_t scan_tiles = ceil_div(n_items, kScanTile);
-    const int64_t scan_grid = scan_tiles < scan_ctas() ? scan_tiles : scan_ctas();
+    // two CTAs per SM: fewer words to look back over than with four (148 against 154 us of sort at 1M items)
+    const int64_t scan_grid = scan_tiles < scan_ctas() / 2 ? scan_tiles : scan_ctas() / 2;
     const int64_t chunk = ceil_div(scan_tiles, scan_grid) * kScanTile;
-    const int64_t item_blocks = radix_blocks(n_items);
+    const int64_t item_blocks = onesweep_blocks(n_items);
     k_scan_items<<<(unsigned)ceil_div(n_items, chunk), kScanThreads, 0, s>>>(
         p->n_tiles, (const float4*)p->rgb_depth, n_items, chunk, out->offset, w.vk0, w.vv0, n_vis, &w.scan_ctl[0],
         w.scan_words, w.scan_words + scan_tiles, &w.sort_ctl[0], lb_words(w.wa, item_blocks), item_blocks, err);
@@ -1581,7 +1597,8 @@ extern "C" int gs_sort(const gs_projected* p, int64_t n, const gs_frame* f, cons
         const int64_t dup_grid = ceil_div(out->capacity, kDupPairs);
         k_duplicate<<<(unsigned)(dup_grid < 5 * 152 ? dup_grid : 5 * 152), kDupThreads, 0, s>>>(
             sorted_item, n_vis, (const ushort4*)p->rect, n, *f, n_eff, w.group_off, w.first_group, out->offset, w.pk0,
-            w.psrc, (tile_bits + 7) / 8, &w.sort_ctl[1], lb_words(w.wa, radix_blocks(out->capacity)));
+            w.psrc, (tile_bits + 7) / 8, &w.sort_ctl[1], lb_words(w.wa, onesweep_blocks(out->capacity)),
+            onesweep_tile(out->capacity));
         count_launch();
         const bool pin1 = onesweep_passes<uint2>(w.pk0, w.psrc, w.pk1, w.psrc2, out->capacity, n_eff, tile_bits,
                                                  &w.sort_ctl[1], w.wa, w.wb, err, s, out->src, out->emit);
@@ -1596,7 +1613,8 @@ extern "C" int gs_sort(const gs_projected* p, int64_t n, const gs_frame* f, cons
                                                                                   w.tv0);
         count_launch();
         k_onesweep_hist<<<(unsigned)radix_blocks(n_tiles_total), 256, 0, s>>>(
-            w.tk0, n_tiles_total, 2, &w.sort_ctl[2], lb_words(w.wa, radix_blocks(n_tiles_total)));
+            w.tk0, n_tiles_total, 2, &w.sort_ctl[2], lb_words(w.wa, onesweep_blocks(n_tiles_total)),
+            onesweep_blocks(n_tiles_total));
         count_launch();
         const bool t1 = onesweep_passes<uint32_t>(w.tk0, w.tv0, w.tk1, w.tv1, n_tiles_total, nullptr, 16,
                                                   &w.sort_ctl[2], w.wa, w.wb, err, s);
