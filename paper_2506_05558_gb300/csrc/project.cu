@@ -1,11 +1,11 @@
-// EWA projection + SH colour (K1). One thread per Gaussian walks its CTA's views (all
-// of them, or a share where there are few Gaussians), so that attributes and SH
-// coefficients are read once: as 128-bit rows, and only for Gaussians that survive a
-// view's cull. The SH rows of a warp's 32 Gaussians pass through shared memory by
+// EWA projection + SH colour (K1). Several views: one thread per Gaussian walks its CTA's
+// views (all of them, or a share where there are few Gaussians), so that attributes and
+// SH coefficients are read once: as 128-bit rows, and only for Gaussians that survive
+// a view's cull. The SH rows of a warp's 32 Gaussians pass through shared memory by
 // asynchronous copies of whole runs: read by each thread from its own row, a warp's
-// load touches 32 lines, and L1 was the bound (71%). 1M Gaussians, SH degree 3,
-// 1080p: one view 52, two 53, eight 197, sixteen views of mixed sizes 670 us (52, 66, 298 and
-// 1185 with a thread per view and Gaussian).
+// load touches 32 lines, and L1 was the bound (71%). 1M Gaussians, SH degree 3, 1080p:
+// two views 53, eight 197, sixteen of mixed sizes 670 us (66, 298 and 1185 with a
+// thread per view and Gaussian). One view has a kernel of its own.
 #include <atomic>
 #include <cstring>
 
@@ -14,61 +14,18 @@
 
 namespace gs {
 
-constexpr int kProjThreads = 128;
-constexpr int64_t kProjCtas = 24 * 152;  // at least four rounds of the CTAs that are resident
-constexpr int kProjPitch = 13;  // float4 from Gaussian to Gaussian: 128-bit loads of 8 lanes hit all banks once
-
-template <int SHD>
-__global__ void __launch_bounds__(kProjThreads, 6) k_project(
-    const float4* __restrict__ mean_opa, const float4* __restrict__ scale, const float4* __restrict__ quat,
-    const float4* __restrict__ sh, int64_t n, const float* __restrict__ filter3d, const gs_camera* __restrict__ cams,
-    const __grid_constant__ gs_frame f, const __grid_constant__ gs_config cfg, int views_per_cta,
-    float2* __restrict__ mean2d, float4* __restrict__ conic_opa, float4* __restrict__ rgb_depth,
-    ushort4* __restrict__ rect, int32_t* __restrict__ n_tiles) {
-    constexpr int NR = (3 * (SHD + 1) * (SHD + 1) + 3) / 4;  // rows of SH coefficients in use
-    __shared__ gs_camera s_cam[GS_MAX_VIEWS];
-    __shared__ __align__(16) float4 s_sh[SHD > 0 ? kProjThreads * kProjPitch : 1];
-    const int v0 = blockIdx.y * views_per_cta, v1 = min(v0 + views_per_cta, f.n_views);
-    for (int i = threadIdx.x; i < (v1 - v0) * (int)(sizeof(gs_camera) / 4); i += kProjThreads)
-        reinterpret_cast<float*>(s_cam)[i] = reinterpret_cast<const float*>(cams + v0)[i];
-    __syncthreads();
-    const unsigned FULL = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    const int64_t g = (int64_t)blockIdx.x * kProjThreads + threadIdx.x;
-    const bool valid = g < n;
-    float4* row = s_sh + (SHD > 0 ? (threadIdx.x - lane) * kProjPitch : 0);  // the warp's rows
-    const float4 mo = valid ? mean_opa[g] : make_float4(0.f, 0.f, 0.f, 0.f);
-    bool have = false, have_sh = false;  // rotation and scales; SH rows
-    float Rq[9], sx = 0.f, sy = 0.f, sz = 0.f, f3 = 1.f;
-#pragma unroll 1
-    for (int v = v0; v < v1; v++) {
-    const int64_t item = (int64_t)v * n + g;
-    const gs_camera& c = s_cam[v - v0];
-    const float x = c.R[0] * mo.x + c.R[1] * mo.y + c.R[2] * mo.z + c.t[0];
-    const float y = c.R[3] * mo.x + c.R[4] * mo.y + c.R[5] * mo.z + c.t[1];
-    const float z = c.R[6] * mo.x + c.R[7] * mo.y + c.R[8] * mo.z + c.t[2];
-    bool keep = valid && z > cfg.near_z;  // false for NaN
-
-    float a = 0.f, b = 0.f, cc = 0.f, det = 0.f, u = 0.f, vv = 0.f, fmip = 1.f;
+// One Gaussian in one view: the 2-D splat and the tiles of its rect.
+struct Splat {
+    float a, b, cc, det, u, vv, fmip;
+    int x0, y0, x1, y1;
+};
+__device__ __forceinline__ bool project_splat(const gs_camera& c, const gs_frame& f, const gs_config& cfg, int v,
+                                              const float4 mo, float x, float y, float z, const float (&Rq)[9], float sx,
+                                              float sy, float sz, float f3, Splat& o) {
+    float a, b, cc, det, u, vv, fmip = 1.f;
     int x0 = 0, y0 = 0, x1 = 0, y1 = 0;
-    if (keep) {
-        if (!have) {
-            have = true;
-            const float4 q4 = quat[g];
-            const float4 s4 = scale[g];
-            const float qi = rsqrtf(q4.x * q4.x + q4.y * q4.y + q4.z * q4.z + q4.w * q4.w);
-            const float qw = q4.x * qi, qx = q4.y * qi, qy = q4.z * qi, qz = q4.w * qi;
-            Rq[0] = 1.f - 2.f * (qy * qy + qz * qz); Rq[1] = 2.f * (qx * qy - qw * qz); Rq[2] = 2.f * (qx * qz + qw * qy);
-            Rq[3] = 2.f * (qx * qy + qw * qz); Rq[4] = 1.f - 2.f * (qx * qx + qz * qz); Rq[5] = 2.f * (qy * qz - qw * qx);
-            Rq[6] = 2.f * (qx * qz - qw * qy); Rq[7] = 2.f * (qy * qz + qw * qx); Rq[8] = 1.f - 2.f * (qx * qx + qy * qy);
-            sx = expf(s4.x); sy = expf(s4.y); sz = expf(s4.z);
-            if (filter3d) {  // 3-D filter: Sigma + v I has scales sqrt(s^2 + v); opacity x prod s / sqrt(s^2 + v)
-                const float fv = filter3d[g];
-                const float px = sqrtf(sx * sx + fv), py = sqrtf(sy * sy + fv), pz = sqrtf(sz * sz + fv);
-                f3 = (sx / px) * (sy / py) * (sz / pz);
-                sx = px; sy = py; sz = pz;
-            }
-        }
+    bool keep;
+    {
         // T = R_cam * Rq * diag(s): camera-space principal axes; Sc = T T^T
         float T[9];
 #pragma unroll
@@ -137,6 +94,144 @@ __global__ void __launch_bounds__(kProjThreads, 6) k_project(
             keep = (x1 - x0) * (y1 - y0) > 0;
         }
     }
+    o = {a, b, cc, det, u, vv, fmip, x0, y0, x1, y1};
+    return keep;
+}
+
+// Rotation and scales of a Gaussian (with the 3-D filter: Sigma + v I has scales sqrt(s^2 + v);
+// opacity x prod s / sqrt(s^2 + v)).
+__device__ __forceinline__ void load_shape(const float4* __restrict__ quat, const float4* __restrict__ scale,
+                                           const float* __restrict__ filter3d, int64_t g, float (&Rq)[9], float& sx,
+                                           float& sy, float& sz, float& f3) {
+    const float4 q4 = quat[g];
+    const float4 s4 = scale[g];
+    const float qi = rsqrtf(q4.x * q4.x + q4.y * q4.y + q4.z * q4.z + q4.w * q4.w);
+    const float qw = q4.x * qi, qx = q4.y * qi, qy = q4.z * qi, qz = q4.w * qi;
+    Rq[0] = 1.f - 2.f * (qy * qy + qz * qz); Rq[1] = 2.f * (qx * qy - qw * qz); Rq[2] = 2.f * (qx * qz + qw * qy);
+    Rq[3] = 2.f * (qx * qy + qw * qz); Rq[4] = 1.f - 2.f * (qx * qx + qz * qz); Rq[5] = 2.f * (qy * qz - qw * qx);
+    Rq[6] = 2.f * (qx * qz - qw * qy); Rq[7] = 2.f * (qy * qz + qw * qx); Rq[8] = 1.f - 2.f * (qx * qx + qy * qy);
+    sx = expf(s4.x); sy = expf(s4.y); sz = expf(s4.z);
+    f3 = 1.f;
+    if (filter3d) {
+        const float fv = filter3d[g];
+        const float px = sqrtf(sx * sx + fv), py = sqrtf(sy * sy + fv), pz = sqrtf(sz * sz + fv);
+        f3 = (sx / px) * (sy / py) * (sz / pz);
+        sx = px; sy = py; sz = pz;
+    }
+}
+
+// Unit view direction: mean - camera centre, centre = -R^T t.
+__device__ __forceinline__ void view_direction(const gs_camera& c, const float4 mo, float& dx, float& dy, float& dz) {
+    const float cx_ = -(c.R[0] * c.t[0] + c.R[3] * c.t[1] + c.R[6] * c.t[2]);
+    const float cy_ = -(c.R[1] * c.t[0] + c.R[4] * c.t[1] + c.R[7] * c.t[2]);
+    const float cz_ = -(c.R[2] * c.t[0] + c.R[5] * c.t[1] + c.R[8] * c.t[2]);
+    dx = mo.x - cx_; dy = mo.y - cy_; dz = mo.z - cz_;
+    const float il = rsqrtf(dx * dx + dy * dy + dz * dz);
+    dx *= il; dy *= il; dz *= il;
+}
+
+// The item's rows, or no tiles where it is culled or its colour or opacity is not finite.
+__device__ __forceinline__ void store_item(bool keep, const Splat& s, float3 rgb, float opa, float z, int64_t item,
+                                           float2* __restrict__ mean2d, float4* __restrict__ conic_opa,
+                                           float4* __restrict__ rgb_depth, ushort4* __restrict__ rect,
+                                           int32_t* __restrict__ n_tiles) {
+    keep = keep && isfinite(rgb.x) && isfinite(rgb.y) && isfinite(rgb.z) && isfinite(opa);
+    if (!keep) {
+        n_tiles[item] = 0;
+        rect[item] = make_ushort4(0, 0, 0, 0);
+        return;
+    }
+    const float idet = 1.f / s.det;
+    mean2d[item] = make_float2(s.u, s.vv);
+    conic_opa[item] = make_float4(s.cc * idet, -s.b * idet, s.a * idet, opa);
+    rgb_depth[item] = make_float4(fmaxf(rgb.x, 0.f), fmaxf(rgb.y, 0.f), fmaxf(rgb.z, 0.f), z);
+    rect[item] = make_ushort4((unsigned short)s.x0, (unsigned short)s.y0, (unsigned short)s.x1, (unsigned short)s.y1);
+    n_tiles[item] = (s.x1 - s.x0) * (s.y1 - s.y0);
+}
+
+// One view: a thread per Gaussian, SH rows read directly, more warps resident than in the
+// form for several views: 65 against 63 us at 1M Gaussians, 197 against 201 at 4M, and
+// 34 against 46 where nine in ten of 2M are culled.
+__global__ void __launch_bounds__(256, 4) k_project_view(
+    const float4* __restrict__ mean_opa, const float4* __restrict__ scale, const float4* __restrict__ quat,
+    const float4* __restrict__ sh, int64_t n, const float* __restrict__ filter3d, const gs_camera* __restrict__ cams,
+    gs_frame f, gs_config cfg, float2* __restrict__ mean2d, float4* __restrict__ conic_opa,
+    float4* __restrict__ rgb_depth, ushort4* __restrict__ rect, int32_t* __restrict__ n_tiles) {
+    __shared__ gs_camera cam_s;
+    if (threadIdx.x < sizeof(gs_camera) / 4)
+        reinterpret_cast<float*>(&cam_s)[threadIdx.x] = reinterpret_cast<const float*>(cams)[threadIdx.x];
+    __syncthreads();
+    const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (g >= n) return;
+    const gs_camera& c = cam_s;
+    const float4 mo = mean_opa[g];
+    const float x = c.R[0] * mo.x + c.R[1] * mo.y + c.R[2] * mo.z + c.t[0];
+    const float y = c.R[3] * mo.x + c.R[4] * mo.y + c.R[5] * mo.z + c.t[1];
+    const float z = c.R[6] * mo.x + c.R[7] * mo.y + c.R[8] * mo.z + c.t[2];
+    bool keep = z > cfg.near_z;  // false for NaN
+    Splat s = {};
+    float f3 = 1.f;
+    if (keep) {
+        float Rq[9], sx, sy, sz;
+        load_shape(quat, scale, filter3d, g, Rq, sx, sy, sz, f3);
+        keep = project_splat(c, f, cfg, 0, mo, x, y, z, Rq, sx, sy, sz, f3, s);
+    }
+    float3 rgb = make_float3(0.f, 0.f, 0.f);
+    float opa = 0.f;
+    if (keep) {
+        float dx, dy, dz, Y[16];
+        view_direction(c, mo, dx, dy, dz);
+        sh_eval_basis(cfg.sh_degree, dx, dy, dz, Y);
+        rgb = sh_color(sh + 12 * g, cfg.sh_degree, Y);
+        opa = f3 * s.fmip / (1.f + expf(-mo.w));
+    }
+    store_item(keep, s, rgb, opa, z, g, mean2d, conic_opa, rgb_depth, rect, n_tiles);
+}
+
+constexpr int kProjThreads = 128;
+// Views share a CTA as far as that leaves one round of the resident CTAs: 200K Gaussians
+// in 4 and 8 views 37 and 59 us; 44 and 63 with at least four rounds.
+constexpr int64_t kProjCtas = 6 * 152;
+constexpr int kProjPitch = 13;  // float4 from Gaussian to Gaussian: 128-bit loads of 8 lanes hit all banks once
+
+template <int SHD>
+__global__ void __launch_bounds__(kProjThreads, 6) k_project(
+    const float4* __restrict__ mean_opa, const float4* __restrict__ scale, const float4* __restrict__ quat,
+    const float4* __restrict__ sh, int64_t n, const float* __restrict__ filter3d, const gs_camera* __restrict__ cams,
+    const __grid_constant__ gs_frame f, const __grid_constant__ gs_config cfg, int views_per_cta,
+    float2* __restrict__ mean2d, float4* __restrict__ conic_opa, float4* __restrict__ rgb_depth,
+    ushort4* __restrict__ rect, int32_t* __restrict__ n_tiles) {
+    constexpr int NR = (3 * (SHD + 1) * (SHD + 1) + 3) / 4;  // rows of SH coefficients in use
+    __shared__ gs_camera s_cam[GS_MAX_VIEWS];
+    __shared__ __align__(16) float4 s_sh[SHD > 0 ? kProjThreads * kProjPitch : 1];
+    const int64_t g = (int64_t)blockIdx.x * kProjThreads + threadIdx.x;
+    const bool valid = g < n;
+    const float4 mo = valid ? mean_opa[g] : make_float4(0.f, 0.f, 0.f, 0.f);
+    const int v0 = blockIdx.y * views_per_cta, v1 = min(v0 + views_per_cta, f.n_views);
+    for (int i = threadIdx.x; i < (v1 - v0) * (int)(sizeof(gs_camera) / 4); i += kProjThreads)
+        reinterpret_cast<float*>(s_cam)[i] = reinterpret_cast<const float*>(cams + v0)[i];
+    __syncthreads();
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    float4* row = s_sh + (SHD > 0 ? (threadIdx.x - lane) * kProjPitch : 0);  // the warp's rows
+    bool have = false, have_sh = false;  // rotation and scales; SH rows
+    float Rq[9], sx = 0.f, sy = 0.f, sz = 0.f, f3 = 1.f;
+#pragma unroll 1
+    for (int v = v0; v < v1; v++) {
+    const int64_t item = (int64_t)v * n + g;
+    const gs_camera& c = s_cam[v - v0];
+    const float x = c.R[0] * mo.x + c.R[1] * mo.y + c.R[2] * mo.z + c.t[0];
+    const float y = c.R[3] * mo.x + c.R[4] * mo.y + c.R[5] * mo.z + c.t[1];
+    const float z = c.R[6] * mo.x + c.R[7] * mo.y + c.R[8] * mo.z + c.t[2];
+    bool keep = valid && z > cfg.near_z;  // false for NaN
+    Splat s = {};
+    if (keep) {
+        if (!have) {
+            have = true;
+            load_shape(quat, scale, filter3d, g, Rq, sx, sy, sz, f3);
+        }
+        keep = project_splat(c, f, cfg, v, mo, x, y, z, Rq, sx, sy, sz, f3, s);
+    }
     if (SHD > 0) {  // the SH rows of the warp's Gaussians that are listed for the first time
         const unsigned need = __ballot_sync(FULL, keep && !have_sh);
         if (need) {
@@ -158,34 +253,14 @@ __global__ void __launch_bounds__(kProjThreads, 6) k_project(
     float3 rgb = make_float3(0.f, 0.f, 0.f);
     float opa = 0.f;
     if (keep) {
-        // view direction: mean - camera centre, centre = -R^T t
-        const float cx_ = -(c.R[0] * c.t[0] + c.R[3] * c.t[1] + c.R[6] * c.t[2]);
-        const float cy_ = -(c.R[1] * c.t[0] + c.R[4] * c.t[1] + c.R[7] * c.t[2]);
-        const float cz_ = -(c.R[2] * c.t[0] + c.R[5] * c.t[1] + c.R[8] * c.t[2]);
-        float dx = mo.x - cx_, dy = mo.y - cy_, dz = mo.z - cz_;
-        const float il = rsqrtf(dx * dx + dy * dy + dz * dz);
-        dx *= il; dy *= il; dz *= il;
-        float Y[16];
+        float dx, dy, dz, Y[16];
+        view_direction(c, mo, dx, dy, dz);
         // squares rounded by themselves for every degree (not fused where degree 2 alone would allow it)
         sh_eval_basis(SHD, dx, dy, dz, __fmul_rn(dx, dx), __fmul_rn(dy, dy), __fmul_rn(dz, dz), Y);
         rgb = SHD > 0 ? sh_color(row + lane * kProjPitch, SHD, Y) : sh_color(sh + 12 * g, SHD, Y);
-        opa = f3 * fmip / (1.f + expf(-mo.w));
-        keep = isfinite(rgb.x) && isfinite(rgb.y) && isfinite(rgb.z) && isfinite(opa);
-        rgb.x = fmaxf(rgb.x, 0.f); rgb.y = fmaxf(rgb.y, 0.f); rgb.z = fmaxf(rgb.z, 0.f);
+        opa = f3 * s.fmip / (1.f + expf(-mo.w));
     }
-    if (!keep) {
-        if (valid) {
-            n_tiles[item] = 0;
-            rect[item] = make_ushort4(0, 0, 0, 0);
-        }
-        continue;
-    }
-    const float idet = 1.f / det;
-    mean2d[item] = make_float2(u, vv);
-    conic_opa[item] = make_float4(cc * idet, -b * idet, a * idet, opa);
-    rgb_depth[item] = make_float4(rgb.x, rgb.y, rgb.z, z);
-    rect[item] = make_ushort4((unsigned short)x0, (unsigned short)y0, (unsigned short)x1, (unsigned short)y1);
-    n_tiles[item] = (x1 - x0) * (y1 - y0);
+    if (valid) store_item(keep, s, rgb, opa, z, item, mean2d, conic_opa, rgb_depth, rect, n_tiles);
     }
 }
 
@@ -293,6 +368,15 @@ extern "C" int gs_project(const gs_gaussians* g, const gs_camera* cams, const gs
     if (!aligned16(g->mean_opa) || !aligned16(g->scale) || !aligned16(g->quat) || !aligned16(g->sh) ||
         !aligned16(out->conic_opa) || !aligned16(out->rgb_depth) || !out->mean2d || !out->rect || !out->n_tiles)
         return GS_ERR_INVALID_ARG;
+    if (f->n_views == 1) {
+        k_project_view<<<(unsigned)ceil_div(g->n, 256), 256, 0, (cudaStream_t)stream>>>(
+            (const float4*)g->mean_opa, (const float4*)g->scale, (const float4*)g->quat, (const float4*)g->sh, g->n,
+            g->filter3d, cams, *f, *cfg, (float2*)out->mean2d, (float4*)out->conic_opa, (float4*)out->rgb_depth,
+            (ushort4*)out->rect, out->n_tiles);
+        count_launch();
+        GS_CUDA_CHECK_LAUNCH();
+        return GS_OK;
+    }
     // all views in one CTA, unless that leaves fewer CTAs than kProjCtas
     const int64_t blocks = ceil_div(g->n, kProjThreads), total = blocks * f->n_views;
     const int per = (int)(total / kProjCtas < 1 ? 1 : total / kProjCtas < f->n_views ? total / kProjCtas : f->n_views);
