@@ -15,7 +15,7 @@
 // global memory in sorted order). Element counts are read from device memory, so the
 // whole sort is enqueued without a host sync and can be captured in a CUDA
 // graph. The reduce-then-scan scan and radix sort below serve the library's
-// other compactions and sorts (spawning, anchors).
+// other compactions and sorts (anchors).
 #include "common.cuh"
 
 namespace gs {
