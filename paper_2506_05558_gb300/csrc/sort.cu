@@ -884,17 +884,22 @@ __device__ __forceinline__ uint2 look_back_cta2(const uint64_t* wa, const uint64
 // slot (exclusive sum of n_tiles in item order: each item's pairs occupy offset[item]
 // .. offset[item] + n_tiles - 1, so that the adjoint's per-item runs of the Gaussians
 // of one view are adjacent), the visible items with their depth keys in item order,
-// their count, the keys' digit counts and the zeroed words of the sort's first pass.
+// their count, the keys' digit counts, the zeroed words of the sort's first pass and
+// empty tile ranges.
 // Chunks and look-back as in k_scan_single, with a word for each of the two sums.
+// SINGLE: a chunk is one tile of 2048 items, read and scanned once.
 // 8M items: 77 us against 72 + 32 + 19 for two scans and a histogram of the keys; the
 // depths' 16-byte stride alone reads 128 MB.
+template <bool SINGLE>
 __global__ void __launch_bounds__(kScanThreads) k_scan_items(const int32_t* __restrict__ n_tiles,
                                                              const float4* __restrict__ rgb_depth, int64_t n,
                                                              int64_t chunk, uint32_t* __restrict__ offset,
                                                              uint32_t* __restrict__ key, uint32_t* __restrict__ val,
                                                              uint32_t* __restrict__ n_vis, ScanCtl* ctl,
                                                              uint64_t* words_v, uint64_t* words_t, SortCtl* sort,
-                                                             LbWords sort_words, int64_t sort_tiles, int32_t* err) {
+                                                             LbWords sort_words, int64_t sort_tiles,
+                                                             uint32_t* __restrict__ range, int64_t n_range,
+                                                             int32_t* err) {
     constexpr int kPad = kScanTile + kScanTile / 32;
     __shared__ uint32_t s_t[kPad];  // tiles of each item, then its first slot
     __shared__ uint32_t s_v[kPad];  // visible items before it (top bit: visible itself)
@@ -903,38 +908,46 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_items(const int32_t* __re
     if (threadIdx.x == 0) s_tile = atomicAdd(&ctl->ticket, 1u);
     for (int p = 0; p < kMaxPasses; p++) s_h[p][threadIdx.x] = 0;
     for (int64_t t = blockIdx.x; t < sort_tiles; t += gridDim.x) lb_zero(sort_words, t);
+    for (int64_t i = (int64_t)blockIdx.x * kScanThreads + threadIdx.x; i < n_range; i += (int64_t)gridDim.x * kScanThreads)
+        range[i] = 0;
     __syncthreads();
     const int64_t c = s_tile, c0 = c * chunk, c1 = min(c0 + chunk, n);  // c < gridDim.x = chunks
-    uint32_t vis = 0, sum = 0;
-    for (int64_t i0 = c0; i0 < c1; i0 += kScanTile) {
-        int32_t t[kScanItems];
-#pragma unroll
-        for (int k = 0; k < kScanItems; k++) {
-            const int64_t i = i0 + k * kScanThreads + threadIdx.x;
-            t[k] = i < c1 ? (int32_t)load_now((const uint32_t*)n_tiles + i) : 0;
-        }
-#pragma unroll
-        for (int k = 0; k < kScanItems; k++) {
-            vis += t[k] > 0;
-            sum += max(t[k], 0);
-        }
-    }
-    uint32_t unused;
-    const uint32_t agg_v = block_exclusive_scan<kScanThreads>(vis, unused);
-    const uint32_t agg_t = block_exclusive_scan<kScanThreads>(sum, unused);
+    uint32_t agg_v = 0, agg_t = 0;
     uint2 run = make_uint2(0, 0);
-    if (threadIdx.x == 0) {
-        lb_store(words_v + c, (c == 0 ? kLbPre : kLbAgg) | agg_v);
-        lb_store(words_t + c, (c == 0 ? kLbPre : kLbAgg) | agg_t);
-    }
-    if (c > 0) {
-        run = look_back_cta2<kScanThreads>(words_v, words_t, c, err);
+    auto look = [&]() {  // publishes the chunk's sums and finds those of the chunks before it
         if (threadIdx.x == 0) {
-            lb_store(words_v + c, kLbPre | (uint32_t)(run.x + agg_v));
-            lb_store(words_t + c, kLbPre | (uint32_t)(run.y + agg_t));
+            lb_store(words_v + c, (c == 0 ? kLbPre : kLbAgg) | agg_v);
+            lb_store(words_t + c, (c == 0 ? kLbPre : kLbAgg) | agg_t);
         }
+        if (c > 0) {
+            run = look_back_cta2<kScanThreads>(words_v, words_t, c, err);
+            if (threadIdx.x == 0) {
+                lb_store(words_v + c, kLbPre | (uint32_t)(run.x + agg_v));
+                lb_store(words_t + c, kLbPre | (uint32_t)(run.y + agg_t));
+            }
+        }
+        if (threadIdx.x == 0 && c1 >= n) *n_vis = run.x + agg_v;
+    };
+    if constexpr (!SINGLE) {
+        uint32_t vis = 0, sum = 0;
+        for (int64_t i0 = c0; i0 < c1; i0 += kScanTile) {
+            int32_t t[kScanItems];
+#pragma unroll
+            for (int k = 0; k < kScanItems; k++) {
+                const int64_t i = i0 + k * kScanThreads + threadIdx.x;
+                t[k] = i < c1 ? (int32_t)load_now((const uint32_t*)n_tiles + i) : 0;
+            }
+#pragma unroll
+            for (int k = 0; k < kScanItems; k++) {
+                vis += t[k] > 0;
+                sum += max(t[k], 0);
+            }
+        }
+        uint32_t unused;
+        agg_v = block_exclusive_scan<kScanThreads>(vis, unused);
+        agg_t = block_exclusive_scan<kScanThreads>(sum, unused);
+        look();
     }
-    if (threadIdx.x == 0 && c1 >= n) *n_vis = run.x + agg_v;
     for (int64_t t0 = c0; t0 < c1; t0 += kScanTile) {
         uint32_t vis_bits = 0;
         uint32_t own[kScanItems];  // tiles of the items this thread writes out, then their depth bits
@@ -963,6 +976,11 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_items(const int32_t* __re
         uint32_t rv, rt;
         const uint32_t gv = block_exclusive_scan<kScanThreads>(tv, rv);
         const uint32_t gt = block_exclusive_scan<kScanThreads>(tt, rt);
+        if constexpr (SINGLE) {
+            agg_v = gv;
+            agg_t = gt;
+            look();
+        }
         rv += run.x;
         rt += run.y;
 #pragma unroll
@@ -1562,8 +1580,8 @@ extern "C" int gs_sort(const gs_projected* p, int64_t n, const gs_frame* f, cons
         GS_CUDA_CHECK_LAUNCH();
         return GS_OK;
     }
-    cudaMemsetAsync(out->range, 0, sizeof(uint32_t) * 2 * n_tiles_total, s);
     if (n_items == 0) {
+        cudaMemsetAsync(out->range, 0, sizeof(uint32_t) * 2 * n_tiles_total, s);
         k_no_pairs<<<1, 1, 0, s>>>(out->count, out->status);
         count_launch();
         GS_CUDA_CHECK_LAUNCH();
@@ -1572,13 +1590,16 @@ extern "C" int gs_sort(const gs_projected* p, int64_t n, const gs_frame* f, cons
     cudaMemsetAsync(w.misc, 0, w.zero_bytes, s);
     // 1. emission slots, and the visible items (in item order) with their depth keys
     const int64_t scan_tiles = ceil_div(n_items, kScanTile);
-    // two CTAs per SM: fewer words to look back over than with four (148 against 154 us of sort at 1M items)
-    const int64_t scan_grid = scan_tiles < scan_ctas() / 2 ? scan_tiles : scan_ctas() / 2;
-    const int64_t chunk = ceil_div(scan_tiles, scan_grid) * kScanTile;
+    // two CTAs per SM: fewer words to look back over than with four (148 against 154 us of sort at 1M
+    // items); a tile each where that is enough (84 against 86 us at 200K)
+    const int64_t scan_tiles_per = scan_tiles <= scan_ctas() / 2 ? 1 : ceil_div(scan_tiles, scan_ctas() / 2);
+    const int64_t chunk = scan_tiles_per * kScanTile;
     const int64_t item_blocks = onesweep_blocks(n_items);
-    k_scan_items<<<(unsigned)ceil_div(n_items, chunk), kScanThreads, 0, s>>>(
+    const auto scan_items = scan_tiles_per == 1 ? k_scan_items<true> : k_scan_items<false>;
+    scan_items<<<(unsigned)ceil_div(n_items, chunk), kScanThreads, 0, s>>>(
         p->n_tiles, (const float4*)p->rgb_depth, n_items, chunk, out->offset, w.vk0, w.vv0, n_vis, &w.scan_ctl[0],
-        w.scan_words, w.scan_words + scan_tiles, &w.sort_ctl[0], lb_words(w.wa, item_blocks), item_blocks, err);
+        w.scan_words, w.scan_words + scan_tiles, &w.sort_ctl[0], lb_words(w.wa, item_blocks), item_blocks,
+        out->range, 2 * n_tiles_total, err);
     count_launch();
     // 2. stable sort of visible items by depth bits
     const bool in1 = onesweep_passes<uint32_t>(w.vk0, w.vv0, w.vk1, w.vv1, n_items, n_vis, 32, &w.sort_ctl[0], w.wa,
