@@ -22,6 +22,7 @@
 // captured into one CUDA graph and replayed without host work.
 #include <cooperative_groups.h>
 #include <mutex>
+#include <type_traits>
 
 #include "common.cuh"
 
@@ -669,10 +670,12 @@ __global__ void __launch_bounds__(128) k_ba_reduce(const double* __restrict__ pa
 
 // The current state's robust cost from the points' costs: sums of 32 points in
 // order, then eight contiguous segments of those in order (an order of its own,
-// whatever the chunks are); warps 1 to 8 of the solving CTA.
+// whatever the chunks are); eight warps of the solving CTA, none of those that
+// back-substitute at the same time.
 __device__ double ba_cost_sum(const double* __restrict__ cost, int64_t P, double* s_part /* [8] */) {
     const int64_t n32 = ceil_div(P, 32), seg = (n32 + 7) / 8;
-    const int w = (int)(threadIdx.x >> 5) - 1, lane = threadIdx.x & 31;  // warps 1 to 8
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int w = (warp & 3) == 3 ? -1 : (warp / 4 - 1) * 3 + (warp & 3);  // warps 4-6, 8-10, 12, 13
     if (w >= 0 && w < 8) {
         const int64_t g0 = w * seg, g1 = min(n32, g0 + seg);
         double a = 0.0;
@@ -749,13 +752,34 @@ __device__ __forceinline__ void ba_retract_entry(const float* Rt, const double* 
 //     takes column k + 1 from its owners - who publish it updated by the columns
 //     before k - applies column k, publishes it and divides, while the others apply
 //     column k to the columns from k + 2;
-//   - one barrier per column.
-// The triangular solves run in one warp: row i's dot product is summed by a fixed
-// tree over lanes, whose sum reaches every lane. 43 x 43: 88 -> 72 us.
-constexpr int kBaSolveThreads = 512;
+//   - one barrier per column among these;
+//   - warp 11 follows them without the barrier: row k of L and of L y = rhs need the
+//     columns before k only, so forward substitution ends with the factorisation. A row
+//     takes it as long as a column takes the others (1040 cycles alone, 1200 beside two
+//     warps of owners; beside three, with four in the other quarters, 1240).
+// A row's dot product is summed by a fixed tree over lanes (xor 16, 8, 4, 2, 1). Back
+// substitution is a chain of rows through that tree from the newest term, always in lane
+// 0, to its root; the tree's other branches end one row earlier, so three helping warps
+// on the other quarters sum them a row ahead and hand them over in shared memory: seven
+// dependent operations a row and no shuffles, 715 cycles against 1000. Branches in a row
+// cost more than the operations that they leave out (levels without terms: 200 cycles a
+// row), hence rows of up to 32 and of more terms as loops of their own.
+// 43 x 43: 88 -> 72 us with both substitutions in one warp after the factorisation, 50 us
+// like this (init 2.5, columns 25, back substitution 14.5, trial cameras and cost 5).
+constexpr int kBaSolveThreads = 480;
+constexpr int kBaForward = 11;  // the substituting warp
 constexpr int kBaEntries = kBaMaxNc * (kBaMaxNc + 1) / 2;
-constexpr int kBaOwners = kBaSolveThreads / 4 * 3;  // the warps whose number is not a multiple of 4
+constexpr int kBaOwners = 320;  // warps 1-3, 5-7, 9, 10, 13, 14: three entries a thread, two warps beside warp 11
 constexpr int kBaPerThread = (kBaEntries + kBaOwners - 1) / kBaOwners;
+
+// Values handed from warp to warp of the solving CTA: the value itself tells whether it
+// is there, an empty place holds a signalling NaN, which no FP64 operation returns. The
+// warps of a CTA all run, so a wait ends; it is bounded all the same.
+constexpr int kBaEmpty = 0x7ff45a5a;  // its high word
+constexpr int kBaWaits = 1 << 16;
+__device__ __forceinline__ double ba_look(const double* place) { return *reinterpret_cast<const volatile double*>(place); }
+__device__ __forceinline__ bool ba_empty(double v) { return __double2hiint(v) == kBaEmpty; }
+__device__ __forceinline__ void ba_hand(double* place, double v) { *reinterpret_cast<volatile double*>(place) = v; }
 
 __global__ void __launch_bounds__(kBaSolveThreads) k_ba_solve(const double* __restrict__ tot,
                                                                const double* __restrict__ cost, int64_t P, int F,
@@ -765,26 +789,31 @@ __global__ void __launch_bounds__(kBaSolveThreads) k_ba_solve(const double* __re
                                                                double* __restrict__ dc, double* __restrict__ cost_cur,
                                                                float* __restrict__ poses_t, float* __restrict__ fl_t,
                                                                int* __restrict__ fail) {
-    __shared__ double U[kBaMaxNc][kBaMaxNc + 1];  // published columns, unscaled: row k holds column k's rows k..
-    __shared__ double L[kBaMaxNc][kBaMaxNc + 1];  // unit lower triangle
-    __shared__ double y[kBaMaxNc], s_rhs[kBaMaxNc];
+    __shared__ double U[kBaMaxNc][kBaMaxNc + 2];  // published columns, unscaled: row k holds column k's rows k..
+    __shared__ double L[kBaMaxNc][kBaMaxNc + 2];  // unit lower triangle
+    __shared__ double y[kBaMaxNc], s_rhs[kBaMaxNc], s_z[kBaMaxNc];
+    __shared__ double s_branch[kBaMaxNc][5];  // back substitution: sums of a row's tree beside its newest term's path
     __shared__ double s_dinv[kBaMaxNc];
     __shared__ double s_part[8];
     __shared__ int s_bad;
     const int nc = ba_nc(F), nup = ba_nup(nc);
     const int tid = threadIdx.x, lane = tid & 31;
     if (tid == 0) s_bad = 0;
-    if (tid < nc) s_rhs[tid] = tot[nup + nc + tid];
+    if (tid < nc) {
+        s_rhs[tid] = tot[nup + nc + tid];
+        y[tid] = s_dinv[tid] = __hiloint2double(kBaEmpty, 0);
+    }
+    if (tid < nc * 5) s_branch[0][tid] = tid < (nc - 2) * 5 ? __hiloint2double(kBaEmpty, 0) : 0.0;  // (row nc - 2: one term)
     const double lam = *lam_p;
     double a[kBaPerThread];
     int ei[kBaPerThread], ej[kBaPerThread];  // row and column of each entry, column -1: none
 #pragma unroll
     for (int s = 0; s < kBaPerThread; s++) {
         const int warp = tid >> 5;
-        const int q = (warp - warp / 4 - 1) * 32 + lane + s * kBaOwners;
+        const int q = (warp - warp / 4 - 1 - (warp > kBaForward)) * 32 + lane + s * kBaOwners;
         ei[s] = ej[s] = -1;
         a[s] = 0.0;
-        if ((warp & 3) && q < nup) {
+        if ((warp & 3) && warp != kBaForward && q < nup) {
             up_ij(q, nc, ej[s], ei[s]);  // upper-triangle entry (column, row)
             a[s] = tot[q];
             if (ei[s] == ej[s]) a[s] += lam * tot[nup + ei[s]] + 1e-9;
@@ -798,78 +827,132 @@ __global__ void __launch_bounds__(kBaSolveThreads) k_ba_solve(const double* __re
         const bool pos = hi >= 0 && (hi | __double2loint(d)) != 0 &&
                          (hi < 0x7ff00000 || (hi == 0x7ff00000 && __double2loint(d) == 0));
         if (!pos) s_bad = 1;
-        s_dinv[k] = pos ? 1.0 / d : 0.0;
+        const double r = pos ? 1.0 / d : 0.0;
+        __threadfence_block();  // the column is there for who sees its pivot
+        ba_hand(&s_dinv[k], r);
     };
     if (tid == 0) pivot(0, U[0][0]);
     __syncthreads();
-    for (int k = 0; k + 1 < nc; k++) {
-        const double dinv = s_dinv[k];
-        if (tid < 32) {  // (the other warps of its quarter own no entry)
-            // column k + 1, rows k + 1 + lane and + 32: the diagonal entry is lane 0's first
-            const int c = k + 1, i0 = c + lane, i1 = i0 + 32;
-            const double p = U[k][c];
-            double v = 0.0, v1 = 0.0;
-            if (i0 < nc) v = U[c][i0] - U[k][i0] * p * dinv;
-            if (i1 < nc) v1 = U[c][i1] - U[k][i1] * p * dinv;
-            if (i0 < nc) U[c][i0] = v;
-            if (i1 < nc) U[c][i1] = v1;
-            if (lane == 0) pivot(c, v);
-        } else {
-#pragma unroll
-            for (int s = 0; s < kBaPerThread; s++)
-                if (ej[s] > k + 1) {
-                    a[s] -= U[k][ei[s]] * U[k][ej[s]] * dinv;
-                    if (ej[s] == k + 2) U[k + 2][ei[s]] = a[s];
-                }
+    const int hi = lane + 32;
+    double y0 = 0.0, y1 = 0.0;  // the substituting warp: lane l holds y_l and y_{l + 32} of L y = rhs
+    auto forward_row = [&](int k, auto wide) {
+        bool wait = true;  // for column k - 1
+        for (int n = 0; n < kBaWaits && wait; n++) wait = __any_sync(0xffffffffu, ba_empty(ba_look(&s_dinv[k - 1])));
+        if (wait) s_bad = 1;
+        __threadfence_block();
+        // no branches: a lane past the row forms the last term again and leaves it out
+        const double rhs = s_rhs[k];
+        const int j0 = min(lane, k - 1), j1 = min(hi, k - 1);
+        const double c0 = __dmul_rn(U[j0][k], s_dinv[j0]);
+        L[k][j0] = c0;
+        double t = __dmul_rn(lane < k ? c0 : 0.0, y0);
+        if constexpr (decltype(wide)::value) {
+            const double c1 = __dmul_rn(U[j1][k], s_dinv[j1]);
+            L[k][j1] = c1;
+            t = __fma_rn(hi < k ? c1 : 0.0, y1, t);
         }
-        __syncthreads();
-    }
-    for (int e = tid; e < nc * nc; e += blockDim.x) {
-        const int k = e / nc, i = e % nc;
-        if (i > k) L[i][k] = U[k][i] * s_dinv[k];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) t = __dadd_rn(t, __shfl_xor_sync(0xffffffffu, t, o));
+        const double v = __dsub_rn(rhs, t);
+        if (lane == k) y0 = v;
+        if (hi == k) y1 = v;
+    };
+    const bool substitutes = tid >> 5 == kBaForward;
+    if (substitutes) {
+        if (lane == 0) y0 = s_rhs[0];
+        int k = 1;
+        for (; k < min(nc, 33); k++) forward_row(k, std::false_type());
+        for (; k < nc; k++) forward_row(k, std::true_type());
+        if (lane < nc) s_z[lane] = y0;
+        if (hi < nc) s_z[hi] = y1;
+    } else {
+        auto column = [&](int k, auto wide) {  // wide: more than 32 rows left
+            const double dinv = s_dinv[k];
+            if (tid < 32) {  // (the other warps of its quarter own no entry)
+                // column k + 1, rows k + 1 + lane and + 32: the diagonal entry is lane 0's first
+                const int c = k + 1, i0 = min(c + lane, nc - 1), i1 = min(i0 + 32, nc - 1);
+                const double p = U[k][c];
+                const double v = U[c][i0] - U[k][i0] * p * dinv;
+                double v1 = 0.0;
+                if constexpr (decltype(wide)::value) v1 = U[c][i1] - U[k][i1] * p * dinv;
+                __syncwarp();
+                if (c + lane < nc) U[c][c + lane] = v;
+                if (decltype(wide)::value && c + lane + 32 < nc) U[c][c + lane + 32] = v1;
+                __syncwarp();
+                if (lane == 0) pivot(c, v);
+            } else {
+#pragma unroll
+                for (int s = 0; s < kBaPerThread; s++)
+                    if (ej[s] > k + 1) {
+                        a[s] -= U[k][ei[s]] * U[k][ej[s]] * dinv;
+                        if (ej[s] == k + 2) U[k + 2][ei[s]] = a[s];
+                    }
+            }
+            asm volatile("bar.sync 1, %0;" ::"n"(kBaSolveThreads - 32) : "memory");  // all but the substituting warp
+        };
+        int k = 0;
+        for (; k + 33 < nc; k++) column(k, std::true_type());
+        for (; k + 1 < nc; k++) column(k, std::false_type());
     }
     __syncthreads();
-    if (tid < 32) {  // L y = rhs, then L^T x = D^-1 y, by one warp; lane l holds y_l and y_{l + 32}
-        const int hi = lane + 32;
-        double y0 = 0.0, y1 = 0.0;
-        // row i's coefficients are loaded while row i - 1 is summed; lanes past the row have 0
-        double c0 = 0.0, c1 = 0.0, b = s_rhs[0];
-        for (int i = 0; i < nc; i++) {
-            double t = c0 * y0;
-            if (i > 32) t += c1 * y1;
-            const double rhs = b;
-            if (i + 1 < nc) {
-                c0 = lane <= i ? L[i + 1][lane] : 0.0;
-                c1 = hi <= i ? L[i + 1][hi] : 0.0;
-                b = s_rhs[i + 1];
-            }
+    if (tid < nc) s_z[tid] = __dmul_rn(s_z[tid], s_dinv[tid]);
+    __syncthreads();
+    // L^T x = D^-1 y, x in y[]: row i's terms j > i start at lane 0 with j = i + 1
+    if (substitutes) {  // every lane the same
+        double x = s_z[nc - 1], z = s_z[nc > 1 ? nc - 2 : 0], l1 = nc > 1 ? L[nc - 1][nc - 2] : 0.0;
+        if (lane == 0) ba_hand(&y[nc - 1], x);
+        auto row = [&](int i, auto wide) {  // wide: more than 32 terms
+            const int next = max(i - 1, 0);
+            double t = __dmul_rn(l1, x);
+            double l33 = 0.0, x33 = 0.0, br[5];
+            if constexpr (decltype(wide)::value) l33 = L[i + 33][i], x33 = ba_look(&y[i + 33]);
+            l1 = L[next + 1][next];
+            const double zi = z;
+            z = s_z[next];
+            bool wait = true;
+            for (int n = 0; n < kBaWaits && wait; n++) {
+                wait = false;
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-            const double v = rhs - t;
-            if (lane == i) y0 = v;
-            if (hi == i) y1 = v;
-        }
-        if (lane < nc) y0 *= s_dinv[lane];
-        if (hi < nc) y1 *= s_dinv[hi];
-        // row i of L^T: its terms j > i start at lane 0 with j = i + 1, so the values that lane
-        // j - i - 1 needs come by shuffles
-        c0 = c1 = 0.0;
-        for (int i = nc - 1; i >= 0; i--) {
-            const int j0 = i + 1 + lane;
-            const double u0 = __shfl_sync(0xffffffffu, y0, j0 & 31), u1 = __shfl_sync(0xffffffffu, y1, j0 & 31);
-            double t = c0 * (j0 < 32 ? u0 : u1);
-            if (i + 33 < nc) t += c1 * u1;
-            if (i > 0) {
-                c0 = j0 - 1 < nc ? L[j0 - 1][i - 1] : 0.0;
-                c1 = j0 + 31 < nc ? L[j0 + 31][i - 1] : 0.0;
-            }
+                for (int s = 0; s < 5; s++) br[s] = ba_look(&s_branch[i][s]);
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-            if (lane == i) y0 -= t;
-            if (hi == i) y1 -= t;
-        }
-        if (lane < nc) y[lane] = y0;
-        if (hi < nc) y[hi] = y1;
+                for (int s = 0; s < 5; s++) wait |= ba_empty(br[s]);
+                wait = __any_sync(0xffffffffu, wait);
+            }
+            if (wait) s_bad = 1;
+            if constexpr (decltype(wide)::value) t = __fma_rn(l33, x33, t);
+#pragma unroll
+            for (int s = 0; s < 5; s++) t = __dadd_rn(t, br[s]);
+            x = __dsub_rn(zi, t);
+            if (lane == 0) ba_hand(&y[i], x);
+        };
+        int i = nc - 2;
+        for (; i >= max(nc - 33, 0); i--) row(i, std::false_type());
+        for (; i >= 0; i--) row(i, std::true_type());
+    } else if (tid < 96) {
+        auto branches = [&](int i, auto wide) {
+            const int m = nc - 1 - i, j = i + 1 + lane;
+            const bool has0 = lane > 0 && lane < m, has1 = decltype(wide)::value && lane > 0 && hi < m;
+            const double l0 = has0 ? L[j][i] : 0.0, l1 = has1 ? L[j + 32][i] : 0.0;
+            double x0 = 0.0, x1 = 0.0;
+            bool wait = true;
+            for (int n = 0; n < kBaWaits && wait; n++) {
+                if (has0) x0 = ba_look(&y[j]);
+                if (has1) x1 = ba_look(&y[j + 32]);
+                wait = __any_sync(0xffffffffu, ba_empty(x0) || ba_empty(x1));
+            }
+            if (wait) s_bad = 1;
+            double t = __dmul_rn(l0, x0);
+            if constexpr (decltype(wide)::value) t = __fma_rn(l1, x1, t);
+#pragma unroll
+            for (int s = 0; s < 5; s++) {
+                const int o = 16 >> s;
+                if (lane == o) ba_hand(&s_branch[i][s], t);
+                if (o > 1) t = __dadd_rn(t, __shfl_xor_sync(0xffffffffu, t, o));
+            }
+        };
+        int i = nc - 3 - (tid >> 5);
+        for (; i >= max(nc - 33, 0); i -= 3) branches(i, std::false_type());
+        for (; i >= 0; i -= 3) branches(i, std::true_type());
     }
     const double total = ba_cost_sum(cost, P, s_part);
     __syncthreads();
