@@ -518,28 +518,62 @@ __global__ void __launch_bounds__(kBaPointsThreads) k_ba_points(const float2* __
 // its threads are dealt densely: the 21 (F - 1) + Nc entries that have an h first,
 // then the others, 512 entries per CTA (two CTAs per chunk at 8 frames: 384, all
 // resident); behind a chunk's last entries two warps take the right-hand side, its
-// products formed by all warps before, and one thread the focal length's, whose
-// chain of adds is F times as long. 8 frames x 6144 points: 190 us with k_ba_points' work in it and
-// the right-hand side in one warp -> 38, k_ba_points 16.
-constexpr int kBaNormalThreads = 512 + 32;
+// products formed by all warps before. The focal length's chain of adds is F times as
+// long as the others' and would come last, at its share of a busy FP64 pipe: CTAs of
+// their own, first in the grid, take it, one thread per chunk. 8 frames x 6144 points:
+// 190 us with k_ba_points' work in it and the right-hand side in one warp -> 38 -> 30,
+// k_ba_points 16.
+constexpr int kBaNormalThreads = 512;
+constexpr int kBaFocalChunks = 8;  // chunks per focal CTA
 
 static size_t ba_normal_smem(int F, int nc) {
-    return sizeof(float) * (2 * kBaChunk * nc * 3 + kBaChunk * F * 17) + sizeof(double) * kBaChunk * (3 + (nc - 1) + nc + F);
+    return sizeof(float) * (2 * kBaChunk * nc * 3 + kBaChunk * F * 17) + sizeof(double) * kBaChunk * (3 + 2 * (nc - 1));
 }
 
 __global__ void __launch_bounds__(kBaNormalThreads) k_ba_normal(BaPoints in, int F, int64_t P,
                                                                 double* __restrict__ partial) {
     extern __shared__ __align__(16) double sm[];
     const int nc = ba_nc(F), nup = ba_nup(nc), tid = threadIdx.x;
-    const bool last = blockIdx.y == gridDim.y - 1;  // this CTA's row has the right-hand side too
-    const int64_t p0 = (int64_t)blockIdx.x * kBaChunk;
+    const int nb = (int)ceil_div(P, kBaChunk), nfocal = (nb + kBaFocalChunks - 1) / kBaFocalChunks;
+    if ((int)blockIdx.x < nfocal) {  // the focal length's right-hand side of these chunks
+        const int c0 = blockIdx.x * kBaFocalChunks, nch = min(kBaFocalChunks, nb - c0), per = kBaChunk * F;
+        double* s_gf = (double*)sm;                     // [32 F][8] gradient terms
+        double* s_kf = s_gf + per * kBaFocalChunks;     // [32][8] K . u
+        for (int i = tid; i < nch * per; i += kBaNormalThreads) {
+            const int64_t o = (int64_t)c0 * per + i;
+            if (o >= P * F) break;
+            const float2 a = *reinterpret_cast<const float2*>(in.J + o * 16 + 6);
+            const float2 b = *reinterpret_cast<const float2*>(in.J + o * 16 + 14);
+            s_gf[i % per * kBaFocalChunks + i / per] = widen(a.x) * widen(a.y) + widen(b.x) * widen(b.y);
+        }
+        for (int i = tid; i < nch * kBaChunk; i += kBaNormalThreads) {
+            const int64_t p = (int64_t)c0 * kBaChunk + i;
+            if (p >= P) break;
+            const float* K = in.K + (p * nc + nc - 1) * 3;
+            const double* u = in.u + p * 3;
+            s_kf[i % kBaChunk * kBaFocalChunks + i / kBaChunk] = widen(K[0]) * u[0] + widen(K[1]) * u[1] + widen(K[2]) * u[2];
+        }
+        __syncthreads();
+        if (tid < nch) {
+            const int np = (int)min((int64_t)kBaChunk, P - (int64_t)(c0 + tid) * kBaChunk);
+            double gc = 0.0, ku = 0.0;
+#pragma unroll 8
+            for (int i = 0; i < np * F; i++) gc += s_gf[i * kBaFocalChunks + tid];
+#pragma unroll 4
+            for (int pt = 0; pt < np; pt++) ku += s_kf[pt * kBaFocalChunks + tid];
+            partial[(int64_t)(c0 + tid) * ba_stride(nc) + nup + nc + nc - 1] = -gc + ku;
+        }
+        return;
+    }
+    const int part = ((int)blockIdx.x - nfocal) / nb, chunk = ((int)blockIdx.x - nfocal) % nb;
+    const bool last = (int)blockIdx.x >= (int)gridDim.x - nb;  // this CTA's row has the right-hand side too
+    const int64_t p0 = (int64_t)chunk * kBaChunk;
     const int np = (int)min((int64_t)kBaChunk, P - p0);
-    double* out = partial + (int64_t)blockIdx.x * ba_stride(nc);
+    double* out = partial + (int64_t)chunk * ba_stride(nc);
     double* s_u = (double*)sm;                       // [32][3]
     double* s_gc = s_u + kBaChunk * 3;               // [32][Nc - 1] gradient terms of the pose parameters
-    double* s_gf = s_gc + kBaChunk * (nc - 1);       // [32][F] and of the focal length
-    double* s_ku = s_gf + kBaChunk * F;              // [32][Nc] K . u
-    float* s_K = (float*)(s_ku + kBaChunk * nc);     // [32][Nc][3]
+    double* s_ku = s_gc + kBaChunk * (nc - 1);       // [32][Nc - 1] K . u
+    float* s_K = (float*)(s_ku + kBaChunk * (nc - 1));  // [32][Nc][3]
     float* s_V = s_K + kBaChunk * nc * 3;            // [32][Nc][3]
     float* s_J = s_V + kBaChunk * nc * 3;            // [32][F][16]
     float* s_w = s_J + kBaChunk * F * 16;            // [32][F]
@@ -554,35 +588,18 @@ __global__ void __launch_bounds__(kBaNormalThreads) k_ba_normal(BaPoints in, int
     if (tid < np * 3) s_u[tid] = in.u[p0 * 3 + tid];
     __syncthreads();
     if (last) {  // the products of the right-hand side, spread over all warps
-        for (int i = tid; i < np * nc; i += kBaNormalThreads) {
-            const int pt = i / nc, c = i % nc, f = c / 6 + 1, a = c % 6;
-            const float* K = s_K + i * 3;
+        for (int i = tid; i < np * (nc - 1); i += kBaNormalThreads) {
+            const int pt = i / (nc - 1), c = i % (nc - 1), f = c / 6 + 1, a = c % 6;
+            const float* K = s_K + (pt * nc + c) * 3;
             const double* u = s_u + pt * 3;
             s_ku[i] = widen(K[0]) * u[0] + widen(K[1]) * u[1] + widen(K[2]) * u[2];
-            if (c < nc - 1) {
-                const float* J = s_J + (pt * F + f) * 16;
-                s_gc[pt * (nc - 1) + c] = widen(J[a]) * widen(J[7]) + widen(J[8 + a]) * widen(J[15]);
-            }
-        }
-        for (int i = tid; i < np * F; i += kBaNormalThreads) {
-            const float* J = s_J + i * 16;
-            s_gf[i] = widen(J[6]) * widen(J[7]) + widen(J[14]) * widen(J[15]);
+            const float* J = s_J + (pt * F + f) * 16;
+            s_gc[i] = widen(J[a]) * widen(J[7]) + widen(J[8 + a]) * widen(J[15]);
         }
         __syncthreads();
     }
-    int q = blockIdx.y * 512 + tid;
+    int q = part * kBaNormalThreads + tid;
     const int q_rhs = (nup + 31) / 32 * 32;  // the warps after the entries
-    if (tid >= 512) {
-        if (last && tid == 512) {
-            double gc = 0.0, ku = 0.0;
-#pragma unroll 8
-            for (int i = 0; i < np * F; i++) gc += s_gf[i];
-#pragma unroll 4
-            for (int pt = 0; pt < np; pt++) ku += s_ku[pt * nc + nc - 1];
-            out[nup + nc + nc - 1] = -gc + ku;
-        }
-        return;
-    }
     if (q >= q_rhs) {
         const int c = q - q_rhs;
         if (c < nc - 1) {
@@ -590,7 +607,7 @@ __global__ void __launch_bounds__(kBaNormalThreads) k_ba_normal(BaPoints in, int
 #pragma unroll 4
             for (int pt = 0; pt < np; pt++) {
                 gc += s_gc[pt * (nc - 1) + c];
-                ku += s_ku[pt * nc + c];
+                ku += s_ku[pt * (nc - 1) + c];
             }
             out[nup + nc + c] = -gc + ku;
         }
@@ -1561,7 +1578,8 @@ extern "C" int gs_ba_lm(const float* obs, int32_t n_frames, int64_t n_points, fl
                              (int)ba_normal_smem(kBaMaxF, kBaMaxNc));
     });
     const int nup = nc * (nc + 1) / 2;
-    const dim3 normal_grid((unsigned)nb, (unsigned)ceil_div(ceil_div(nup, 32) * 32 + nc - 1, 512));
+    const unsigned normal_grid = (unsigned)(ceil_div(nb, kBaFocalChunks) +
+                                            nb * ceil_div(ceil_div(nup, 32) * 32 + nc - 1, kBaNormalThreads));
     const int stride = nc * (nc + 1) / 2 + 2 * nc;
     const float2* ob = (const float2*)obs;
     float4* pts = (float4*)points;
