@@ -277,7 +277,7 @@ typedef struct gs_grads {
 size_t gs_backward_workspace_size(int64_t n, const gs_frame* f, int64_t capacity);
 
 /* Adjoint of project + sort + render_fwd for all views at once.
- *   dL_dcolor  same layout as gs_image.color
+ *   dL_dcolor  same layout as gs_image.color; like the image's buffers it may start at any float
  *   grads      OVERWRITTEN with dL/d(parameters) summed over views
  *   dL_dpose   [n_views][6] OVERWRITTEN: dL/dxi for the left perturbation
  *              T_cw <- exp(xi^) T_cw, xi = (rho, phi) (translation first)

@@ -801,11 +801,12 @@ constexpr int kRowBlocks = 8;  // 8x4 blocks of a tile, one per quad of lanes
 struct RowInfo {
     int view, x, y, W, n_in;  // first pixel; how many of the eight lie in the view
     int64_t pix, plane, color_base;
-    bool vec;                 // all eight lie in the view and 16-byte accesses are aligned
+    bool vec;                 // all eight lie in the view and 16-byte loads are aligned
     float tx0, ty0;           // the tile's first pixel centre
 };
 
-__device__ __forceinline__ RowInfo row_info(const gs_frame& f, int tile) {
+// aligned: the buffers that rows are read from start on 16 bytes.
+__device__ __forceinline__ RowInfo row_info(const gs_frame& f, int tile, bool aligned) {
     RowInfo t;
     t.view = view_of_tile(f, tile);
     const int local = tile - f.tile_base[t.view];
@@ -820,13 +821,13 @@ __device__ __forceinline__ RowInfo row_info(const gs_frame& f, int tile) {
     const int64_t pb = f.pix_base[t.view];
     t.pix = pb + (int64_t)t.y * t.W + t.x;
     t.color_base = 3 * pb + (int64_t)t.y * t.W + t.x;
-    t.vec = t.n_in == kRowPx && ((t.W | (int)pb) & 3) == 0;
+    t.vec = aligned && t.n_in == kRowPx && ((t.W | (int)pb) & 3) == 0;
     t.tx0 = (float)(tx * kFastTile) + 0.5f;
     t.ty0 = (float)(ty * kFastTile) + 0.5f;
     return t;
 }
 
-// A row's eight values from or to memory (aligned: two 16-byte accesses).
+// A row's eight values from memory (aligned: two 16-byte loads).
 template <class T, class V4>
 __device__ __forceinline__ void load_row(const T* __restrict__ p, const RowInfo& t, T (&v)[kRowPx]) {
     if (t.vec) {
@@ -836,19 +837,6 @@ __device__ __forceinline__ void load_row(const T* __restrict__ p, const RowInfo&
 #pragma unroll
         for (int i = 0; i < kRowPx; i++)
             if (i < t.n_in) v[i] = p[i];
-    }
-}
-template <class T, class V4>
-__device__ __forceinline__ void store_row(T* __restrict__ p, const RowInfo& t, const T (&v)[kRowPx]) {
-    if (t.vec) {
-        V4 a, b;
-        a.x = v[0]; a.y = v[1]; a.z = v[2]; a.w = v[3]; b.x = v[4]; b.y = v[5]; b.z = v[6]; b.w = v[7];
-        reinterpret_cast<V4*>(p)[0] = a;
-        reinterpret_cast<V4*>(p)[1] = b;
-    } else {
-#pragma unroll
-        for (int i = 0; i < kRowPx; i++)
-            if (i < t.n_in) p[i] = v[i];
     }
 }
 
@@ -907,7 +895,7 @@ __global__ void __launch_bounds__(32, 16) k_rows_bwd(gs_frame f, gs_config cfg, 
                                                      const float* __restrict__ dL_dcolor, float4* __restrict__ part0,
                                                      float4* __restrict__ part1, float* __restrict__ part2,
                                                      int64_t capacity, const uint32_t* __restrict__ order,
-                                                     uint32_t* counter, int n_tiles) {
+                                                     uint32_t* counter, int n_tiles, bool aligned) {
     __shared__ float2 s_raw_xy[kBwdBatch];  // the next batch's projected rows
     __shared__ float4 s_raw_co[kBwdBatch];
     __shared__ float4 s_raw_rgb[kBwdBatch];
@@ -926,7 +914,7 @@ __global__ void __launch_bounds__(32, 16) k_rows_bwd(gs_frame f, gs_config cfg, 
     }
     for (int tile = next_tile(order, counter, n_tiles, true, &s_item); tile >= 0;
          tile = next_tile(order, counter, n_tiles, false, &s_item)) {
-        const RowInfo ti = row_info(f, tile);
+        const RowInfo ti = row_info(f, tile, aligned);
         const float py = ti.y + 0.5f;
         const uint32_t start = range[2 * tile];
         int nc[kRowPx];
@@ -1313,9 +1301,11 @@ int launch_render_bwd(const gs_projected* p, const gs_pairs* pairs, const gs_fra
     const float* tf = fwd->t_final;
     const int32_t* nc = fwd->n_contrib;
     int64_t cap = pairs->capacity;
+    // a caller's image or gradient may be any slice of a larger buffer; k_rows_bwd alone takes the flag
+    bool aligned = (((uintptr_t)tf | (uintptr_t)nc | (uintptr_t)dL_dcolor) & 15) == 0;
     void* args[] = {&fv, &cv, (void*)&range, (void*)&src, (void*)&emit, (void*)&m2, (void*)&co, (void*)&rd,
                     (void*)&tf, (void*)&nc, (void*)&dL_dcolor, (void*)&part0, (void*)&part1, (void*)&part2,
-                    &cap, (void*)&order, (void*)&counter, &n_tiles};
+                    &cap, (void*)&order, (void*)&counter, &n_tiles, &aligned};
     return launch(L, n_tiles, persistent, args, s);
 }
 }  // namespace gs
