@@ -780,9 +780,12 @@ __global__ void __launch_bounds__(kRadixThreads, 3) k_onesweep_pass(
     }
 }
 
-// Look-back words of one radix pass over at most n_max keys.
+// Look-back words that a radix pass over n_max keys or fewer needs at most: the tiles
+// halve at kFewKeys, so that many keys have more of them than somewhat more keys do, and
+// a workspace sized for the largest sort of several has to hold the others too.
 static int64_t onesweep_words(int64_t n_max) {
-    const int64_t tiles = onesweep_blocks(n_max);
+    const int64_t few = onesweep_blocks(n_max < kFewKeys ? n_max : kFewKeys), all = onesweep_blocks(n_max);
+    const int64_t tiles = few > all ? few : all;
     return 256 * (tiles + 2 * lb_groups(tiles));
 }
 
