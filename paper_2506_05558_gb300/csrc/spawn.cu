@@ -369,14 +369,13 @@ struct SpawnScratch {
     uint32_t* scan;
 };
 
-static SpawnScratch carve_spawn(Carve& c, int W, int H) {
+static SpawnScratch carve_spawn(Carve& c, int64_t pixels, int64_t words) {
     SpawnScratch w;
-    const int64_t n = mask_words(W, H);
-    w.mask = c.take<uint32_t>(n);
-    w.prefix = c.take<uint32_t>(n);
+    w.mask = c.take<uint32_t>(words);
+    w.prefix = c.take<uint32_t>(words);
     w.total = c.take<uint32_t>(1);
-    w.p_l = c.take<float>((size_t)W * H);
-    w.scan = c.take<uint32_t>(scan_popcounts_words(n));
+    w.p_l = c.take<float>(pixels);
+    w.scan = c.take<uint32_t>(scan_popcounts_words(words));
     return w;
 }
 
@@ -435,7 +434,8 @@ extern "C" size_t gs_spawn_workspace_size(int32_t width, int32_t height) {
     if (width <= 0 || height <= 0) return 0;
     const int64_t hw = (int64_t)width * height;
     Carve c{nullptr, 0, 0};
-    carve_spawn(c, width, height);
+    // as many words as a frame one pixel wide has: what this many pixels need in any shape
+    carve_spawn(c, hw, hw);
     c.take<float>(hw);       // gs_spawn_learned: P_s
     c.take<float>(hw / 64);  // gs_spawn_learned: patch sums
     return c.used;
@@ -453,7 +453,7 @@ extern "C" int gs_spawn_propose(const float* image, const float* render, const f
     LogTaps taps;
     if (!make_taps(sc->sigma, &taps)) return GS_ERR_INVALID_ARG;
     Carve c{(char*)ws, 0, ws_bytes};
-    const SpawnScratch w = carve_spawn(c, width, height);
+    const SpawnScratch w = carve_spawn(c, hw, mask_words(width, height));
     if (!ws || !c.ok() || ((uintptr_t)ws & 255)) return GS_ERR_INVALID_ARG;
     if (height > kSpMaxHeight) return GS_ERR_CUDA;
     return spawn_propose(image, render, depth, width, height, cam, sc, out, taps, w, (cudaStream_t)stream);
@@ -557,7 +557,7 @@ extern "C" int gs_spawn_propose_noalloc(const float* image, const float* render,
     // reads (the mask and its prefix counts, P_L where the mask is set, and the
     // scan's words, which the call clears).
     Carve c{(char*)base, 0, sizeof(uint32_t) * kNoAllocWords};
-    const SpawnScratch w = carve_spawn(c, width, height);
+    const SpawnScratch w = carve_spawn(c, hw, mask_words(width, height));
     if (!c.ok()) return GS_ERR_INVALID_ARG;
     return spawn_propose(image, render, depth, width, height, cam, sc, out, taps, w, (cudaStream_t)stream);
 }
@@ -700,7 +700,7 @@ extern "C" int gs_spawn_learned(const float* image, const float* mlp_out, const 
     LogTaps taps;
     if (!make_taps(sc->sigma, &taps)) return GS_ERR_INVALID_ARG;
     Carve c{(char*)ws, 0, ws_bytes};
-    const SpawnScratch w = carve_spawn(c, width, height);
+    const SpawnScratch w = carve_spawn(c, hw, mask_words(width, height));
     float* ps = c.take<float>(hw);
     float* sums = c.take<float>(hw / 64);
     if (!ws || !c.ok() || ((uintptr_t)ws & 255)) return GS_ERR_INVALID_ARG;

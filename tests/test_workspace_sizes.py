@@ -31,3 +31,10 @@ def test_sort_workspace_grows_with_tiles():
     for n, c in ((0, 0), (1000, 5000), (1 << 20, 1 << 20)):
         sizes = [gs.gs_sort_workspace_size(n, gs.frame([(8 * w, 8 * 1024)], 8), c) for w in (1, 500, 1023, 1024, 1025, 1100, 2049)]
         assert sizes == sorted(sizes)
+
+
+def test_spawn_workspace_depends_on_the_pixels_alone():
+    sizes = [gs.gs_spawn_workspace_size(w, h) for w, h in ((1920, 1080), (1080, 1920), (2073600, 1), (1, 2073600), (33, 62836))]
+    assert all(s <= sizes[0] for s in sizes), sizes
+    grow = [gs.gs_spawn_workspace_size(w, h) for w, h in ((1, 1), (31, 1), (1, 32), (64, 64), (65, 64), (31, 4000), (4000, 32))]
+    assert grow == sorted(grow), grow
