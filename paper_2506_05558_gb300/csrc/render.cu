@@ -967,13 +967,18 @@ __global__ void __launch_bounds__(32, 16) k_rows_bwd(gs_frame f, gs_config cfg, 
         // pairs past every pixel's last contributor get a zero partial (their
         // emission slots are summed per Gaussian like all others)
         const uint32_t len = range[2 * tile + 1] - start;
-        for (uint32_t j = (uint32_t)n_list + lane; j < len; j += 32) {
-            const uint32_t e = emit[start + j];
-            if ((int64_t)e < capacity) {
-                part0[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-                part1[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-                part2[e] = 0.f;
-            }
+        constexpr int kZeros = 8;
+        for (uint32_t j0 = (uint32_t)n_list + lane; j0 < len; j0 += 32 * kZeros) {
+            uint32_t e[kZeros];
+#pragma unroll
+            for (int k = 0; k < kZeros; k++) e[k] = j0 + 32 * k < len ? emit[start + j0 + 32 * k] : 0xffffffffu;
+#pragma unroll
+            for (int k = 0; k < kZeros; k++)
+                if ((int64_t)e[k] < capacity) {
+                    part0[e[k]] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    part1[e[k]] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    part2[e[k]] = 0.f;
+                }
         }
         auto fetch = [&](int q, uint32_t idx) {  // entry q's rows on their way to this lane's places
             if (q >= 0) {
