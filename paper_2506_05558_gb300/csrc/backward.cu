@@ -103,8 +103,16 @@ __global__ void __launch_bounds__(32 * kGatherWarps) k_item_partials(
             else if (k + 1 < kGatherRuns) fetch(lo[k + 1 < kGatherRuns ? k + 1 : k], hi[k + 1 < kGatherRuns ? k + 1 : k], win[buf ^ 1]);
             else asm volatile("cp.async.commit_group;" ::: "memory");
             asm volatile("cp.async.wait_group 1;" ::: "memory");
+            Win& s = win[buf];
+            if (base < hi[k]) {  // slots that hold no partial become zeros (each lane those that it fetched)
+                const int cnt = (int)min(hi[k] - base, (uint32_t)kGatherWin);
+                for (int j = lane; j < cnt; j += 32)
+                    if (__float_as_uint(s.c[j]) == kNoPartial) {
+                        s.a[j] = s.b[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        s.c[j] = 0.f;
+                    }
+            }
             __syncwarp();
-            const Win& s = win[buf];
             if (base < hi[k]) {
                 const uint32_t to = min(end, hi[k] - base > kGatherWin ? base + kGatherWin : hi[k]);
                 for (uint32_t q = max(beg, base); q < to; q++) {

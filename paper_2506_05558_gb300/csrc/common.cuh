@@ -77,6 +77,10 @@ __device__ __forceinline__ unsigned lanemask_lt() {
     return m;
 }
 
+// In the last word of a (tile, Gaussian) pair's partial: no pixel composites the pair and
+// its other words are not written. A signalling NaN, which no arithmetic returns.
+constexpr uint32_t kNoPartial = 0x7fa5a5a5u;
+
 // Host-side count of kernels this library has launched (diagnostics).
 void count_launch();
 

@@ -974,11 +974,7 @@ __global__ void __launch_bounds__(32, 16) k_rows_bwd(gs_frame f, gs_config cfg, 
             for (int k = 0; k < kZeros; k++) e[k] = j0 + 32 * k < len ? emit[start + j0 + 32 * k] : 0xffffffffu;
 #pragma unroll
             for (int k = 0; k < kZeros; k++)
-                if ((int64_t)e[k] < capacity) {
-                    part0[e[k]] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    part1[e[k]] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    part2[e[k]] = 0.f;
-                }
+                if ((int64_t)e[k] < capacity) part2[e[k]] = __uint_as_float(kNoPartial);
         }
         auto fetch = [&](int q, uint32_t idx) {  // entry q's rows on their way to this lane's places
             if (q >= 0) {
