@@ -241,6 +241,81 @@ __global__ void __launch_bounds__(TILE * TILE) k_render_fwd(gs_frame f, gs_confi
     }
 }
 
+// Long lists in launches of k_rows_bwd (further down). Its one warp per tile takes 0.116 us
+// for each entry that a pixel composites, with an SM to itself, and k_render_bwd's eight
+// 0.072, so that uneven launches ended with single warps at their longest lists. Tiles
+// with more than kLongMean times the mean list (uniform scenes have up to 4.5 times) go to
+// k_render_bwd, launched to start when the last CTA of k_rows_bwd has started and the
+// registers of the first ones are free: 100k Gaussians over a 720p view and 20k more in
+// 60 x 60 px of it, 901 us without and 604 with it (604 by k_render_bwd for all tiles);
+// 400k in 60 clusters over a 1080p view 386 and 295 (413); 200k all over a 720p view, no
+// long list, 82 and 85. Three CTAs per SM: with two, 400k Gaussians in 200 x 200 px of two
+// 1080p views took 2000 us instead of 1340. Each CTA looks through all ranges, so launches of more than kLongTiles
+// tiles do without: four 1080p views with such clusters take 1.05 to 1.4 times k_render_bwd's time.
+constexpr int kLongMean = 8, kLongTiles = 16384, kLongCtas = 3 * 152;
+constexpr uint32_t kLongMin = 1024;
+__device__ __forceinline__ uint32_t long_list(const int64_t* __restrict__ count, int64_t capacity, float share) {
+    return max(kLongMin, __float2uint_rz(__fmul_rn((float)(uint32_t)min(*count, capacity), share)));
+}
+
+// Launches that overlap: the next one may start when every CTA of this one has called
+// launch_next or ended; wait_for_last returns when the one before has ended.
+__device__ __forceinline__ void launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_last() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// The tiles with long lists, dealt to the CTAs in turn: this CTA's to s_mine; their number.
+constexpr int kLongMine = (kLongTiles / kLongMean + kLongCtas - 1) / kLongCtas;
+template <int NT>
+__device__ __forceinline__ int my_long_tiles(const uint32_t* __restrict__ range, int n_tiles, uint32_t len, int* s_mine) {
+    constexpr int NW = NT / 32, kWords = kLongTiles / 32, kPer = kWords / NT, kAhead = 8;
+    __shared__ unsigned s_mask[kWords];  // a bit per tile
+    __shared__ int s_count[NW], s_n;
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    unsigned any = 0;
+#pragma unroll 1
+    for (int t0 = 0; t0 < kLongTiles; t0 += kAhead * NT) {
+        uint32_t a[kAhead], b[kAhead];
+#pragma unroll
+        for (int k = 0; k < kAhead; k++) {
+            const int t = min(t0 + k * NT + (int)threadIdx.x, n_tiles - 1);
+            a[k] = range[2 * t];
+            b[k] = range[2 * t + 1];
+        }
+#pragma unroll
+        for (int k = 0; k < kAhead; k++) {
+            const int t = t0 + k * NT + threadIdx.x;
+            const unsigned m = __ballot_sync(FULL, t < n_tiles && b[k] - a[k] > len);
+            if (lane == 0) s_mask[t / 32] = m;
+            any |= m;
+        }
+    }
+    if (threadIdx.x == 0) s_n = 0;
+    if (!__syncthreads_or(any != 0)) return 0;
+    // a tile's rank: the long ones of the words before its own, then of its word
+    int mine = 0;
+#pragma unroll
+    for (int k = 0; k < kPer; k++) mine += __popc(s_mask[threadIdx.x * kPer + k]);
+    int rank = mine;  // inclusive over the warp
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(FULL, rank, o);
+        if (lane >= o) rank += u;
+    }
+    if (lane == 31) s_count[w] = rank;
+    __syncthreads();
+    rank -= mine;
+    for (int q = 0; q < w; q++) rank += s_count[q];
+    for (int k = 0; k < kPer; k++)
+        for (unsigned m = s_mask[threadIdx.x * kPer + k]; m; m &= m - 1, rank++)
+            if (rank % (int)gridDim.x == (int)blockIdx.x) {
+                const int i = atomicAdd(&s_n, 1);
+                if (i < kLongMine) s_mine[i] = 32 * ((int)threadIdx.x * kPer + k) + __ffs(m) - 1;
+            }
+    __syncthreads();
+    return min(s_n, kLongMine);
+}
+
 // Compositing adjoint. Per pixel (one lane) and Gaussian, back to front: the
 // transmittance in front of it, dL/dalpha and from it the two scalars that all
 // nine gradient terms of the (tile, Gaussian) pair are built from - dpow =
@@ -251,7 +326,9 @@ __global__ void __launch_bounds__(TILE * TILE) k_render_fwd(gs_frame f, gs_confi
 // each and combine in a fixed order: about a third fewer instructions per hit.
 constexpr int kBwdHits = 8;  // hits per table flush (4 lanes per hit, 8 pixels each)
 
-template <int TILE, int BB>
+//
+// LONG: the tiles with long lists of a launch whose others k_rows_bwd takes, beside it.
+template <int TILE, int BB, bool LONG = false>
 __global__ void __launch_bounds__(TILE * TILE) k_render_bwd(gs_frame f, gs_config cfg,
                                                             const uint32_t* __restrict__ range,
                                                             const uint32_t* __restrict__ src,
@@ -265,7 +342,8 @@ __global__ void __launch_bounds__(TILE * TILE) k_render_bwd(gs_frame f, gs_confi
                                                             float4* __restrict__ part0, float4* __restrict__ part1,
                                                             float* __restrict__ part2, int64_t capacity,
                                                             const uint32_t* __restrict__ order, uint32_t* counter,
-                                                            int n_tiles) {
+                                                            int n_tiles, const int64_t* __restrict__ count,
+                                                            float share) {
     constexpr int NT = Geom<TILE>::kThreads;
     constexpr int NW = Geom<TILE>::kWarps;
     __shared__ float2 s_xy[BB];
@@ -284,8 +362,11 @@ __global__ void __launch_bounds__(TILE * TILE) k_render_bwd(gs_frame f, gs_confi
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const float inv_log2e = 1.f / kLog2e;
-    for (int tile = next_tile(order, counter, n_tiles, true, &s_item); tile >= 0;
-         tile = next_tile(order, counter, n_tiles, false, &s_item)) {
+    __shared__ int s_mine[LONG ? kLongMine : 1];
+    int left = LONG ? my_long_tiles<NT>(range, n_tiles, long_list(count, capacity, share), s_mine) : 0;
+    auto next_long = [&]() { return left > 0 ? s_mine[--left] : -1; };
+    for (int tile = LONG ? next_long() : next_tile(order, counter, n_tiles, true, &s_item); tile >= 0;
+         tile = LONG ? next_long() : next_tile(order, counter, n_tiles, false, &s_item)) {
         const TileInfo ti = tile_info<TILE>(f, tile);
         const WarpBlock wb = warp_block(ti);
         const float px = ti.px + 0.5f, py = ti.py + 0.5f;
@@ -305,16 +386,12 @@ __global__ void __launch_bounds__(TILE * TILE) k_render_bwd(gs_frame f, gs_confi
         if (lane == 0) atomicMax(&s_max, warp_nc);
         __syncthreads();
         const int n_list = s_max;
-        // pairs past every pixel's last contributor get a zero partial (their
-        // emission slots are summed per Gaussian like all others)
+        // pairs past every pixel's last contributor: their emission slots are gathered per
+        // Gaussian like all others
         const uint32_t len = range[2 * tile + 1] - start;
         for (uint32_t j = (uint32_t)n_list + threadIdx.x; j < len; j += NT) {
             const uint32_t e = emit[start + j];
-            if ((int64_t)e < capacity) {
-                part0[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-                part1[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-                part2[e] = 0.f;
-            }
+            if ((int64_t)e < capacity) part2[e] = __uint_as_float(kNoPartial);
         }
         // gS = sum over channels of dL/dC_ch times the colour composited behind the
         // current Gaussian plus the background seen through T_final: dL/dalpha needs
@@ -455,6 +532,8 @@ __global__ void __launch_bounds__(TILE * TILE) k_render_bwd(gs_frame f, gs_confi
         }
         __syncthreads();  // shared buffers are reused by the next tile
     }
+    // this launch ends no sooner than the one that it overlaps: those after it wait for both
+    if (LONG && blockIdx.x == 0) wait_for_last();
 }
 
 // ---------------------------------------------------------------------------
@@ -789,10 +868,14 @@ __global__ void __launch_bounds__(kFwdThreads) k_blocks_fwd(gs_frame f, gs_confi
 // warps per SM, which registers and the block sums in shared memory allow). Of
 // this the exact block test took 3.05 to 2.89 ms, batches of 32 instead of 64
 // with the next rows on their way 2.42, the cheaper staging 2.33. One warp per
-// tile needs many tiles: at 920 tiles 115 against 98 us, at 1840 tiles 134 against
-// 150.
+// tile needs many tiles, more of them in several small views, whose full tiles in the
+// middle come round at the same SMs: 200k Gaussians in seven 320x240 views (2,100
+// tiles) 714 against 499 us, in one of 960x640 (2,400) 91 against 93, in four of 480x400
+// (3,000) 267 against 286, in one of 1100x720 (3,105) 85 against 96, in eight of 400x320
+// (4,000) 493 against 508, in one of 1280x720 (3,600) 82 against 101: from 20 tiles per SM,
+// a quarter more than are resident.
 // ---------------------------------------------------------------------------
-constexpr int kBwdMinTiles = 1408;
+constexpr int kBwdMinTiles = 20 * 152;
 constexpr int kRowPx = 8;      // pixels of a lane
 constexpr int kRowBlocks = 8;  // 8x4 blocks of a tile, one per quad of lanes
 
@@ -895,7 +978,8 @@ __global__ void __launch_bounds__(32, 16) k_rows_bwd(gs_frame f, gs_config cfg, 
                                                      const float* __restrict__ dL_dcolor, float4* __restrict__ part0,
                                                      float4* __restrict__ part1, float* __restrict__ part2,
                                                      int64_t capacity, const uint32_t* __restrict__ order,
-                                                     uint32_t* counter, int n_tiles, bool aligned) {
+                                                     uint32_t* counter, int n_tiles,
+                                                     const int64_t* __restrict__ count, float share, bool aligned) {
     __shared__ float2 s_raw_xy[kBwdBatch];  // the next batch's projected rows
     __shared__ float4 s_raw_co[kBwdBatch];
     __shared__ float4 s_raw_rgb[kBwdBatch];
@@ -907,6 +991,7 @@ __global__ void __launch_bounds__(32, 16) k_rows_bwd(gs_frame f, gs_config cfg, 
     const int lane = threadIdx.x, blk = lane >> 2;
     const float inv_log2e = 1.f / kLog2e;
     const float alpha_min = cfg.alpha_min;
+    if (share > 0.f) launch_next();
     if (lane == 0) {
         BwdRow none = {};
         none.o = -INFINITY;  // times 2^0: below any alpha_min
@@ -914,9 +999,10 @@ __global__ void __launch_bounds__(32, 16) k_rows_bwd(gs_frame f, gs_config cfg, 
     }
     for (int tile = next_tile(order, counter, n_tiles, true, &s_item); tile >= 0;
          tile = next_tile(order, counter, n_tiles, false, &s_item)) {
+        const uint32_t start = range[2 * tile], len = range[2 * tile + 1] - start;
+        if (share > 0.f && len > long_list(count, capacity, share)) continue;  // k_render_bwd's
         const RowInfo ti = row_info(f, tile, aligned);
         const float py = ti.y + 0.5f;
-        const uint32_t start = range[2 * tile];
         int nc[kRowPx];
         f32x2 xs[kRowPx / 2], T2[kRowPx / 2], S2[kRowPx / 2], nr[kRowPx / 2], ng[kRowPx / 2], nb[kRowPx / 2];
         {
@@ -964,9 +1050,8 @@ __global__ void __launch_bounds__(32, 16) k_rows_bwd(gs_frame f, gs_config cfg, 
         // contributor (pixels outside the view have none and keep that test on)
         const int n_plain = ti.n_in == kRowPx ? nc_low : 0;
         const int n_all = __reduce_min_sync(FULL, (unsigned)n_plain);
-        // pairs past every pixel's last contributor get a zero partial (their
-        // emission slots are summed per Gaussian like all others)
-        const uint32_t len = range[2 * tile + 1] - start;
+        // pairs past every pixel's last contributor: their emission slots are gathered per
+        // Gaussian like all others
         constexpr int kZeros = 8;
         for (uint32_t j0 = (uint32_t)n_list + lane; j0 < len; j0 += 32 * kZeros) {
             uint32_t e[kZeros];
@@ -1197,13 +1282,22 @@ static int default_fwd_batch(int tile, int n_tiles) {
 }
 static int default_bwd_batch(int tile) { return tile == 32 ? 32 : tile == 16 ? 64 : 128; }
 
-static int launch(const RenderLaunch& L, int n_tiles, bool persistent, void** args, cudaStream_t s) {
-    int grid = n_tiles;
+// overlap: the launch starts when the one before allows it (launch_next), not when that ends.
+static int launch(const RenderLaunch& L, int grid, bool persistent, void** args, cudaStream_t s, bool overlap = false) {
     if (persistent) {
         const int pg = persistent_grid(L.fn, L.threads);
-        grid = n_tiles < pg ? n_tiles : pg;
+        grid = grid < pg ? grid : pg;
     }
-    if (cudaLaunchKernel(L.fn, dim3(grid), dim3(L.threads), args, 0, s) != cudaSuccess) {
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(grid);
+    lc.blockDim = dim3(L.threads);
+    lc.stream = s;
+    lc.attrs = &at;
+    lc.numAttrs = overlap ? 1 : 0;
+    if (cudaLaunchKernelExC(&lc, L.fn, args) != cudaSuccess) {
         (void)cudaGetLastError();
         return GS_ERR_CUDA;
     }
@@ -1296,6 +1390,9 @@ int launch_render_bwd(const gs_projected* p, const gs_pairs* pairs, const gs_fra
     const uint32_t* range = pairs->range;
     const uint32_t* src = pairs->src;
     const uint32_t* emit = pairs->emit;
+    const int64_t* count = pairs->count;
+    const bool rows = L.fn == (const void*)k_rows_bwd;
+    float share = rows && count && n_tiles <= kLongTiles ? kLongMean / (float)n_tiles : 0.f;  // (without a count: none long)
     const float2* m2 = (const float2*)p->mean2d;
     const float4* co = (const float4*)p->conic_opa;
     const float4* rd = (const float4*)p->rgb_depth;
@@ -1306,7 +1403,9 @@ int launch_render_bwd(const gs_projected* p, const gs_pairs* pairs, const gs_fra
     bool aligned = (((uintptr_t)tf | (uintptr_t)nc | (uintptr_t)dL_dcolor) & 15) == 0;
     void* args[] = {&fv, &cv, (void*)&range, (void*)&src, (void*)&emit, (void*)&m2, (void*)&co, (void*)&rd,
                     (void*)&tf, (void*)&nc, (void*)&dL_dcolor, (void*)&part0, (void*)&part1, (void*)&part2,
-                    &cap, (void*)&order, (void*)&counter, &n_tiles, &aligned};
-    return launch(L, n_tiles, persistent, args, s);
+                    &cap, (void*)&order, (void*)&counter, &n_tiles, (void*)&count, &share, &aligned};
+    const int rc = launch(L, n_tiles, persistent, args, s);
+    if (rc != GS_OK || !(share > 0.f)) return rc;
+    return launch({(const void*)k_render_bwd<kFastTile, 64, true>, kFastTile * kFastTile}, kLongCtas, false, args, s, true);
 }
 }  // namespace gs
