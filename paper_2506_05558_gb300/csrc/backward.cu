@@ -572,16 +572,18 @@ __global__ void __launch_bounds__(256) k_pose_reduce(const float* __restrict__ p
 
 int launch_render_bwd(const gs_projected* p, const gs_pairs* pairs, const gs_frame* f, const gs_config* cfg,
                       const gs_image* fwd, const float* dL_dcolor, float4* part0, float4* part1, float* part2,
-                      uint32_t* counter, cudaStream_t s);
+                      uint32_t* counter, uint8_t* again /* [n_tiles] */, cudaStream_t s);
 
 struct BwdWs {
     float4 *part0, *part1;
     float *part2, *pose_part;
     float4* rec;
     uint32_t* counter;
+    uint8_t* again;
 };
 
-static BwdWs carve_bwd(char* base, size_t cap, int64_t n, int n_views, int64_t capacity, size_t* used) {
+static BwdWs carve_bwd(char* base, size_t cap, int64_t n, const gs_frame& f, int64_t capacity, size_t* used) {
+    const int n_views = f.n_views;
     Carve c{base, 0, cap};
     BwdWs w;
     w.part0 = c.take<float4>(capacity);
@@ -589,6 +591,7 @@ static BwdWs carve_bwd(char* base, size_t cap, int64_t n, int n_views, int64_t c
     w.part2 = c.take<float>(capacity);
     w.pose_part = c.take<float>((size_t)n_views * ceil_div(n, kPBThreads) * 6);
     w.counter = c.take<uint32_t>(4);
+    w.again = c.take<uint8_t>(f.tile_base[n_views]);
     w.rec = c.take<float4>((size_t)n_views * n * 3);  // per-item sums of the pair partials
     *used = c.used;
     return w;
@@ -601,7 +604,7 @@ using namespace gs;
 extern "C" size_t gs_backward_workspace_size(int64_t n, const gs_frame* f, int64_t capacity) {
     if (!f || n < 0 || capacity < 0) return 0;
     size_t used = 0;
-    carve_bwd(nullptr, 0, n, f->n_views, capacity, &used);
+    carve_bwd(nullptr, 0, n, *f, capacity, &used);
     return used;
 }
 
@@ -617,11 +620,11 @@ extern "C" int gs_composite_bwd(const gs_projected* p, const gs_pairs* pairs, co
                                 void* ws, size_t ws_bytes, void* stream) {
     if (!p || !pairs || !fwd || !dL_dcolor || n < 0 || check_bwd_common(f, cfg) != GS_OK) return GS_ERR_INVALID_ARG;
     size_t need = 0;
-    BwdWs w = carve_bwd((char*)ws, ws_bytes, n, f->n_views, pairs->capacity, &need);
+    BwdWs w = carve_bwd((char*)ws, ws_bytes, n, *f, pairs->capacity, &need);
     if (!ws || ws_bytes < need || ((uintptr_t)ws & 255)) return GS_ERR_INVALID_ARG;
     if (n == 0) return GS_OK;
     return launch_render_bwd(p, pairs, f, cfg, fwd, dL_dcolor, w.part0, w.part1, w.part2, w.counter,
-                             (cudaStream_t)stream);
+                             w.again, (cudaStream_t)stream);
 }
 
 extern "C" int gs_project_bwd(const gs_gaussians* g, const gs_camera* cams, const gs_projected* p,
@@ -632,7 +635,7 @@ extern "C" int gs_project_bwd(const gs_gaussians* g, const gs_camera* cams, cons
     if (!grads->mean_opa || !grads->scale || !grads->quat || !grads->sh || !grads->visible) return GS_ERR_INVALID_ARG;
     if (g->n > 0 && (!pairs->offset || !pairs->status)) return GS_ERR_INVALID_ARG;
     size_t need = 0;
-    BwdWs w = carve_bwd((char*)ws, ws_bytes, g->n, f->n_views, pairs->capacity, &need);
+    BwdWs w = carve_bwd((char*)ws, ws_bytes, g->n, *f, pairs->capacity, &need);
     if (!ws || ws_bytes < need || ((uintptr_t)ws & 255)) return GS_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     if (g->n == 0) {

@@ -327,7 +327,8 @@ __device__ __forceinline__ int my_long_tiles(const uint32_t* __restrict__ range,
 constexpr int kBwdHits = 8;  // hits per table flush (4 lanes per hit, 8 pixels each)
 
 //
-// LONG: the tiles with long lists of a launch whose others k_rows_bwd takes, beside it.
+// LONG: the tiles of a launch of k_rows_bwd that are not for it: those with long lists,
+// beside it, and when it has ended those that it marked (again: a byte per tile).
 template <int TILE, int BB, bool LONG = false>
 __global__ void __launch_bounds__(TILE * TILE) k_render_bwd(gs_frame f, gs_config cfg,
                                                             const uint32_t* __restrict__ range,
@@ -343,7 +344,7 @@ __global__ void __launch_bounds__(TILE * TILE) k_render_bwd(gs_frame f, gs_confi
                                                             float* __restrict__ part2, int64_t capacity,
                                                             const uint32_t* __restrict__ order, uint32_t* counter,
                                                             int n_tiles, const int64_t* __restrict__ count,
-                                                            float share) {
+                                                            float share, uint8_t* again) {
     constexpr int NT = Geom<TILE>::kThreads;
     constexpr int NW = Geom<TILE>::kWarps;
     __shared__ float2 s_xy[BB];
@@ -363,8 +364,37 @@ __global__ void __launch_bounds__(TILE * TILE) k_render_bwd(gs_frame f, gs_confi
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const float inv_log2e = 1.f / kLog2e;
     __shared__ int s_mine[LONG ? kLongMine : 1];
-    int left = LONG ? my_long_tiles<NT>(range, n_tiles, long_list(count, capacity, share), s_mine) : 0;
-    auto next_long = [&]() { return left > 0 ? s_mine[--left] : -1; };
+    __shared__ unsigned s_again[NW];
+    int mine = 0, word = NW;
+    unsigned bits = 0;
+    int64_t at = 0, seen = blockIdx.x;  // tiles at + i gridDim.x are in s_again; the next to look at
+    if (LONG && share > 0.f) mine = my_long_tiles<NT>(range, n_tiles, long_list(count, capacity, share), s_mine);
+    auto next_long = [&]() {
+        if (mine > 0) return s_mine[--mine];
+        for (;;) {
+            if (bits) {
+                const int i = 32 * (word - 1) + __ffs(bits) - 1;
+                bits &= bits - 1;
+                return (int)(at + (int64_t)i * gridDim.x);
+            }
+            if (word < NW) {
+                bits = s_again[word++];
+                continue;
+            }
+            if (seen >= n_tiles) return -1;
+            wait_for_last();  // every CTA comes here: this launch ends no sooner than the one that it overlaps
+            __syncthreads();
+            at = seen;
+            const int64_t t = at + (int64_t)threadIdx.x * gridDim.x;
+            unsigned is = 0;
+            if (t < n_tiles) asm volatile("ld.relaxed.gpu.global.u8 %0, [%1];" : "=r"(is) : "l"(again + t) : "memory");
+            const unsigned m = __ballot_sync(FULL, is != 0);
+            if (lane == 0) s_again[w] = m;
+            __syncthreads();
+            seen += (int64_t)NT * gridDim.x;
+            word = 0;
+        }
+    };
     for (int tile = LONG ? next_long() : next_tile(order, counter, n_tiles, true, &s_item); tile >= 0;
          tile = LONG ? next_long() : next_tile(order, counter, n_tiles, false, &s_item)) {
         const TileInfo ti = tile_info<TILE>(f, tile);
@@ -532,8 +562,6 @@ __global__ void __launch_bounds__(TILE * TILE) k_render_bwd(gs_frame f, gs_confi
         }
         __syncthreads();  // shared buffers are reused by the next tile
     }
-    // this launch ends no sooner than the one that it overlaps: those after it wait for both
-    if (LONG && blockIdx.x == 0) wait_for_last();
 }
 
 // ---------------------------------------------------------------------------
@@ -965,6 +993,12 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_al
 // not touch enters with alpha = 0, which leaves its state as it is and adds zeros,
 // so one select per pixel is all the predication there is. The next batch's
 // projected rows are on their way (cp.async) while this one is worked on.
+//
+// A product with that zero is NaN where the other factor is not finite: a pixel whose
+// gradient is infinite or NaN would spoil the sums of every Gaussian listed for its
+// block, not of those that it composites. k_render_bwd has selects for that and does
+// tiles with such a sum once more (a look at the pixels' gradients cost 3% of this kernel's
+// speed, a second form of its loop 5%).
 constexpr int kBwdBatch = 32;
 
 __global__ void __launch_bounds__(32, 16) k_rows_bwd(gs_frame f, gs_config cfg, const uint32_t* __restrict__ range,
@@ -979,7 +1013,8 @@ __global__ void __launch_bounds__(32, 16) k_rows_bwd(gs_frame f, gs_config cfg, 
                                                      float4* __restrict__ part1, float* __restrict__ part2,
                                                      int64_t capacity, const uint32_t* __restrict__ order,
                                                      uint32_t* counter, int n_tiles,
-                                                     const int64_t* __restrict__ count, float share, bool aligned) {
+                                                     const int64_t* __restrict__ count, float share,
+                                                     uint8_t* __restrict__ again, bool aligned) {
     __shared__ float2 s_raw_xy[kBwdBatch];  // the next batch's projected rows
     __shared__ float4 s_raw_co[kBwdBatch];
     __shared__ float4 s_raw_rgb[kBwdBatch];
@@ -991,7 +1026,7 @@ __global__ void __launch_bounds__(32, 16) k_rows_bwd(gs_frame f, gs_config cfg, 
     const int lane = threadIdx.x, blk = lane >> 2;
     const float inv_log2e = 1.f / kLog2e;
     const float alpha_min = cfg.alpha_min;
-    if (share > 0.f) launch_next();
+    launch_next();
     if (lane == 0) {
         BwdRow none = {};
         none.o = -INFINITY;  // times 2^0: below any alpha_min
@@ -1000,6 +1035,7 @@ __global__ void __launch_bounds__(32, 16) k_rows_bwd(gs_frame f, gs_config cfg, 
     for (int tile = next_tile(order, counter, n_tiles, true, &s_item); tile >= 0;
          tile = next_tile(order, counter, n_tiles, false, &s_item)) {
         const uint32_t start = range[2 * tile], len = range[2 * tile + 1] - start;
+        if (lane == 0) again[tile] = 0;
         if (share > 0.f && len > long_list(count, capacity, share)) continue;  // k_render_bwd's
         const RowInfo ti = row_info(f, tile, aligned);
         const float py = ti.y + 0.5f;
@@ -1139,8 +1175,7 @@ __global__ void __launch_bounds__(32, 16) k_rows_bwd(gs_frame f, gs_config cfg, 
                         // the same decisions as the forward pass: listed before this pixel's last
                         // contributor, exponent <= 0, alpha >= alpha_min; na = -alpha, or 0. Alpha
                         // clamped at alpha_max passes no gradient to the exponent or opacity (nog);
-                        // selects (not products with 0) keep a non-finite 2^e outside the Gaussian
-                        // out of the sums.
+                        // selects keep a non-finite 2^e outside the Gaussian out of the sums.
                         float na[2], nog[2], m[2], dx[2], d[2];
 #pragma unroll
                         for (int h = 0; h < 2; h++) {
@@ -1229,6 +1264,7 @@ __global__ void __launch_bounds__(32, 16) k_rows_bwd(gs_frame f, gs_config cfg, 
                 part0[em] = make_float4(a[0], a[1], -0.5f * a[4], -a[5]);
                 part1[em] = make_float4(-0.5f * a[2], e.o > 0.f ? a[8] / e.o : 0.f, a[3], a[6]);
                 part2[em] = a[7];
+                if (!(fabsf(a[8]) < INFINITY)) again[tile] = 1;
             }
             __syncwarp();  // rows, lists and sums are rewritten by the next batch
         }
@@ -1375,7 +1411,7 @@ extern "C" int gs_render_fwd_count(const gs_projected* p, const gs_pairs* pairs,
 namespace gs {
 int launch_render_bwd(const gs_projected* p, const gs_pairs* pairs, const gs_frame* f, const gs_config* cfg,
                       const gs_image* fwd, const float* dL_dcolor, float4* part0, float4* part1, float* part2,
-                      uint32_t* counter, cudaStream_t s) {
+                      uint32_t* counter, uint8_t* again, cudaStream_t s) {
     if (!render_args_ok(f, cfg)) return GS_ERR_INVALID_ARG;
     int n_tiles = f->tile_base[f->n_views];
     if (n_tiles == 0) return GS_OK;
@@ -1403,9 +1439,9 @@ int launch_render_bwd(const gs_projected* p, const gs_pairs* pairs, const gs_fra
     bool aligned = (((uintptr_t)tf | (uintptr_t)nc | (uintptr_t)dL_dcolor) & 15) == 0;
     void* args[] = {&fv, &cv, (void*)&range, (void*)&src, (void*)&emit, (void*)&m2, (void*)&co, (void*)&rd,
                     (void*)&tf, (void*)&nc, (void*)&dL_dcolor, (void*)&part0, (void*)&part1, (void*)&part2,
-                    &cap, (void*)&order, (void*)&counter, &n_tiles, (void*)&count, &share, &aligned};
+                    &cap, (void*)&order, (void*)&counter, &n_tiles, (void*)&count, &share, (void*)&again, &aligned};
     const int rc = launch(L, n_tiles, persistent, args, s);
-    if (rc != GS_OK || !(share > 0.f)) return rc;
+    if (rc != GS_OK || !rows) return rc;
     return launch({(const void*)k_render_bwd<kFastTile, 64, true>, kFastTile * kFastTile}, kLongCtas, false, args, s, true);
 }
 }  // namespace gs
