@@ -33,7 +33,7 @@ constexpr int kBaMaxNc = 6 * (kBaMaxF - 1) + 1;  // 43 camera parameters
 
 __device__ __forceinline__ int ba_nc(int F) { return 6 * (F - 1) + 1; }
 __device__ __forceinline__ int ba_nup(int nc) { return nc * (nc + 1) / 2; }
-__device__ __forceinline__ int ba_stride(int nc) { return ba_nup(nc) + 2 * nc + 1; }  // S_up | H diag | rhs | cost
+__device__ __forceinline__ int ba_stride(int nc) { return ba_nup(nc) + 2 * nc; }  // S_up | H diag | rhs
 
 struct BaObs {
     float r[2], e, w;
@@ -1142,7 +1142,7 @@ static BaWs carve_ba(char* base, size_t cap, int F, int64_t P, size_t* used) {
     w.poses_t = c.take<float>(12 * kBaMaxF);
     w.fl_t = c.take<float>(4);
     w.pts_t = c.take<float4>(P);
-    w.partial = c.take<double>(nb * (nc * (nc + 1) / 2 + 2 * nc + 1));
+    w.partial = c.take<double>(nb * (nc * (nc + 1) / 2 + 2 * nc));
     w.trial_partial = c.take<double>(nt);
     w.pt.K = c.take<float>(P * nc * 3);
     w.pt.V = c.take<float>(P * nc * 3);
@@ -1154,7 +1154,7 @@ static BaWs carve_ba(char* base, size_t cap, int F, int64_t P, size_t* used) {
     w.pt.w = c.take<float>(n);
     w.dc = c.take<double>(kBaMaxNc);
     w.cost_cur = c.take<double>(1);
-    w.tot = c.take<double>(nc * (nc + 1) / 2 + 2 * nc + 1);
+    w.tot = c.take<double>(nc * (nc + 1) / 2 + 2 * nc);
     w.trial_total = c.take<double>(1);
     w.thr = c.take<float>(1);
     w.iter = c.take<int>(1);
@@ -1616,7 +1616,7 @@ extern "C" int gs_ba_lm(const float* obs, int32_t n_frames, int64_t n_points, fl
         count_launch();
         k_ba_normal<<<normal_grid, kBaNormalThreads, ba_normal_smem(F, nc), s>>>(w.pt, F, P, w.partial);
         count_launch();
-        k_ba_reduce<<<(unsigned)ceil_div(stride, 16), dim3(16, 8), 0, s>>>(w.partial, nb, stride + 1, stride, w.tot);
+        k_ba_reduce<<<(unsigned)ceil_div(stride, 16), dim3(16, 8), 0, s>>>(w.partial, nb, stride, stride, w.tot);
         count_launch();
         k_ba_solve<<<1, kBaSolveThreads, 0, s>>>(w.tot, w.pt.cost, P, F, lam, poses, fl, w.dc, w.cost_cur, w.poses_t,
                                                  w.fl_t, w.fail);

@@ -151,7 +151,7 @@ __device__ __forceinline__ void quat_rotation(float qw, float qx, float qy, floa
 // DV > 0 (at most DV views): each view's colour gradient is kept in shared
 // memory and the SH-coefficient sums are formed after the view loop (the view
 // direction computed again there), so their 3 (d + 1)^2 accumulators are not
-// live across it: 128 registers (a few bytes spilled), four CTAs per SM;
+// live across it: 128 registers (92 bytes spilled at degree 3), four CTAs per SM;
 // DV = 0: accumulated view by view.
 constexpr int kPBDeferViews = 16;
 

@@ -218,49 +218,49 @@ __global__ void __launch_bounds__(kProjThreads, 6) k_project(
     float Rq[9], sx = 0.f, sy = 0.f, sz = 0.f, f3 = 1.f;
 #pragma unroll 1
     for (int v = v0; v < v1; v++) {
-    const int64_t item = (int64_t)v * n + g;
-    const gs_camera& c = s_cam[v - v0];
-    const float x = c.R[0] * mo.x + c.R[1] * mo.y + c.R[2] * mo.z + c.t[0];
-    const float y = c.R[3] * mo.x + c.R[4] * mo.y + c.R[5] * mo.z + c.t[1];
-    const float z = c.R[6] * mo.x + c.R[7] * mo.y + c.R[8] * mo.z + c.t[2];
-    bool keep = valid && z > cfg.near_z;  // false for NaN
-    Splat s = {};
-    if (keep) {
-        if (!have) {
-            have = true;
-            load_shape(quat, scale, filter3d, g, Rq, sx, sy, sz, f3);
-        }
-        keep = project_splat(c, f, cfg, v, mo, x, y, z, Rq, sx, sy, sz, f3, s);
-    }
-    if (SHD > 0) {  // the SH rows of the warp's Gaussians that are listed for the first time
-        const unsigned need = __ballot_sync(FULL, keep && !have_sh);
-        if (need) {
-            const float4* first = sh + 12 * (g - lane);
-#pragma unroll
-            for (int k = 0; k < NR; k++) {
-                const int gl = (32 * k + lane) / NR, r = (32 * k + lane) % NR;
-                if ((need >> gl) & 1u)
-                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
-                                     (uint32_t)__cvta_generic_to_shared(row + gl * kProjPitch + r)),
-                                 "l"(first + 12 * gl + r)
-                                 : "memory");
+        const int64_t item = (int64_t)v * n + g;
+        const gs_camera& c = s_cam[v - v0];
+        const float x = c.R[0] * mo.x + c.R[1] * mo.y + c.R[2] * mo.z + c.t[0];
+        const float y = c.R[3] * mo.x + c.R[4] * mo.y + c.R[5] * mo.z + c.t[1];
+        const float z = c.R[6] * mo.x + c.R[7] * mo.y + c.R[8] * mo.z + c.t[2];
+        bool keep = valid && z > cfg.near_z;  // false for NaN
+        Splat s = {};
+        if (keep) {
+            if (!have) {
+                have = true;
+                load_shape(quat, scale, filter3d, g, Rq, sx, sy, sz, f3);
             }
-            asm volatile("cp.async.wait_all;" ::: "memory");
-            __syncwarp();
-            have_sh |= keep;
+            keep = project_splat(c, f, cfg, v, mo, x, y, z, Rq, sx, sy, sz, f3, s);
         }
-    }
-    float3 rgb = make_float3(0.f, 0.f, 0.f);
-    float opa = 0.f;
-    if (keep) {
-        float dx, dy, dz, Y[16];
-        view_direction(c, mo, dx, dy, dz);
-        // squares rounded by themselves for every degree (not fused where degree 2 alone would allow it)
-        sh_eval_basis(SHD, dx, dy, dz, __fmul_rn(dx, dx), __fmul_rn(dy, dy), __fmul_rn(dz, dz), Y);
-        rgb = SHD > 0 ? sh_color(row + lane * kProjPitch, SHD, Y) : sh_color(sh + 12 * g, SHD, Y);
-        opa = f3 * s.fmip / (1.f + expf(-mo.w));
-    }
-    if (valid) store_item(keep, s, rgb, opa, z, item, mean2d, conic_opa, rgb_depth, rect, n_tiles);
+        if (SHD > 0) {  // the SH rows of the warp's Gaussians that are listed for the first time
+            const unsigned need = __ballot_sync(FULL, keep && !have_sh);
+            if (need) {
+                const float4* first = sh + 12 * (g - lane);
+#pragma unroll
+                for (int k = 0; k < NR; k++) {
+                    const int gl = (32 * k + lane) / NR, r = (32 * k + lane) % NR;
+                    if ((need >> gl) & 1u)
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                                         (uint32_t)__cvta_generic_to_shared(row + gl * kProjPitch + r)),
+                                     "l"(first + 12 * gl + r)
+                                     : "memory");
+                }
+                asm volatile("cp.async.wait_all;" ::: "memory");
+                __syncwarp();
+                have_sh |= keep;
+            }
+        }
+        float3 rgb = make_float3(0.f, 0.f, 0.f);
+        float opa = 0.f;
+        if (keep) {
+            float dx, dy, dz, Y[16];
+            view_direction(c, mo, dx, dy, dz);
+            // squares rounded by themselves for every degree (not fused where degree 2 alone would allow it)
+            sh_eval_basis(SHD, dx, dy, dz, __fmul_rn(dx, dx), __fmul_rn(dy, dy), __fmul_rn(dz, dz), Y);
+            rgb = SHD > 0 ? sh_color(row + lane * kProjPitch, SHD, Y) : sh_color(sh + 12 * g, SHD, Y);
+            opa = f3 * s.fmip / (1.f + expf(-mo.w));
+        }
+        if (valid) store_item(keep, s, rgb, opa, z, item, mean2d, conic_opa, rgb_depth, rect, n_tiles);
     }
 }
 

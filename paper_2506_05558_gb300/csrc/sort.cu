@@ -486,16 +486,14 @@ __device__ __forceinline__ uint2 load_now2(const uint2* p) {
     return v;
 }
 
-// Exclusive scan of load(0..n-1) into out[0..n_max) (positions at or past the
-// valid count n = min(n_max, *n_dev) get the total), total -> *total. Each CTA
+// Exclusive scan of load(0..n-1) into out[0..n), total -> *total. Each CTA
 // takes one contiguous chunk: it sums the chunk, publishes the sum, looks
 // back over the earlier chunks (all CTAs of the grid run at once, so the walk
 // covers at most a round or two of the CTA-wide window), then scans the chunk
 // tile by tile (its second read mostly hits L2).
 template <class Load>
-__global__ void __launch_bounds__(kScanThreads) k_scan_single(Load load, uint32_t* __restrict__ out, int64_t n_max,
-                                                              const uint32_t* n_dev, int64_t chunk,
-                                                              ScanCtl* ctl, uint64_t* words, uint32_t* total,
+__global__ void __launch_bounds__(kScanThreads) k_scan_single(Load load, uint32_t* __restrict__ out, int64_t n,
+                                                              int64_t chunk, ScanCtl* ctl, uint64_t* words, uint32_t* total,
                                                               int32_t* err) {
     // each tile passes through shared memory so that global loads and stores
     // are coalesced while each thread scans 8 consecutive values (one padding
@@ -506,18 +504,16 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_single(Load load, uint32_
     __syncthreads();
     const int64_t c = s_tile;
     const int64_t c0 = c * chunk;
-    if (c0 >= n_max) return;  // uniform over the CTA
-    const int64_t c1 = min(c0 + chunk, n_max);
-    const int64_t n = valid_count(n_max, n_dev);
-    const int64_t cv = min(c1, n);  // end of the valid part of the chunk
+    if (c0 >= n) return;  // uniform over the CTA
+    const int64_t c1 = min(c0 + chunk, n);
     uint32_t sum = 0;
 #pragma unroll 2
-    for (int64_t i0 = c0; i0 < cv; i0 += kScanTile) {
+    for (int64_t i0 = c0; i0 < c1; i0 += kScanTile) {
         uint32_t part[kScanItems];
 #pragma unroll
         for (int k = 0; k < kScanItems; k++) {
             const int64_t i = i0 + k * kScanThreads + threadIdx.x;
-            part[k] = i < cv ? load(i) : 0u;
+            part[k] = i < c1 ? load(i) : 0u;
         }
 #pragma unroll
         for (int k = 0; k < kScanItems; k++) sum += part[k];
@@ -533,12 +529,12 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_single(Load load, uint32_
         run = look_back_cta<kScanThreads>(words, c, err);
         if (threadIdx.x == 0) lb_store(mine, kLbPre | (uint32_t)(run + agg));
     }
-    if (threadIdx.x == 0 && total && c1 >= n_max) *total = run + agg;
+    if (threadIdx.x == 0 && total && c1 >= n) *total = run + agg;
     for (int64_t t0 = c0; t0 < c1; t0 += kScanTile) {
 #pragma unroll
         for (int k = 0; k < kScanItems; k++) {
             const int i = k * kScanThreads + threadIdx.x;
-            s_v[i + (i >> 5)] = t0 + i < cv ? load(t0 + i) : 0u;
+            s_v[i + (i >> 5)] = t0 + i < c1 ? load(t0 + i) : 0u;
         }
         __syncthreads();
         uint32_t v[kScanItems];
@@ -584,14 +580,13 @@ static int64_t scan_ctas() {
 }
 
 template <class Load>
-static void scan_single(Load load, uint32_t* out, int64_t n_max, const uint32_t* n_dev, uint32_t* total,
-                        ScanCtl* ctl, uint64_t* words, int32_t* err, cudaStream_t s) {
-    const int64_t tiles = ceil_div(n_max, kScanTile);
+static void scan_single(Load load, uint32_t* out, int64_t n, uint32_t* total, ScanCtl* ctl, uint64_t* words,
+                        int32_t* err, cudaStream_t s) {
+    const int64_t tiles = ceil_div(n, kScanTile);
     if (tiles == 0) return;
     const int64_t g = tiles < scan_ctas() ? tiles : scan_ctas();
     const int64_t chunk = ceil_div(tiles, g) * kScanTile;
-    k_scan_single<<<(unsigned)ceil_div(n_max, chunk), kScanThreads, 0, s>>>(load, out, n_max, n_dev, chunk, ctl, words,
-                                                                           total, err);
+    k_scan_single<<<(unsigned)ceil_div(n, chunk), kScanThreads, 0, s>>>(load, out, n, chunk, ctl, words, total, err);
     count_launch();
 }
 
@@ -604,7 +599,7 @@ size_t scan_popcounts_words(int64_t n) { return 64 + 2 * ceil_div(n, kScanTile);
 
 int32_t* scan_popcounts(const uint32_t* words, uint32_t* out, int64_t n, uint32_t* total, uint32_t* ws, cudaStream_t s) {
     int32_t* err = (int32_t*)ws + 32;
-    scan_single(LoadPopcount{words}, out, n, nullptr, total, (ScanCtl*)ws, (uint64_t*)(ws + 64), err, s);
+    scan_single(LoadPopcount{words}, out, n, total, (ScanCtl*)ws, (uint64_t*)(ws + 64), err, s);
     return err;
 }
 
@@ -905,7 +900,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_items(const int32_t* __re
                                                              int32_t* err) {
     constexpr int kPad = kScanTile + kScanTile / 32;
     __shared__ uint32_t s_t[kPad];  // tiles of each item, then its first slot
-    __shared__ uint32_t s_v[kPad];  // visible items before it (top bit: visible itself)
+    __shared__ uint32_t s_v[kPad];  // visible items before it
     __shared__ uint32_t s_h[kMaxPasses][256];
     __shared__ uint32_t s_tile;
     if (threadIdx.x == 0) s_tile = atomicAdd(&ctl->ticket, 1u);
