@@ -16,7 +16,14 @@ from .raster import Rasterizer, copy_config
 
 FWD_BATCHES = {8: (64, 128, 256), 16: (64, 128, 256), 32: (128, 256)}
 BWD_BATCHES = {8: (64, 128, 256), 16: (32, 64, 128), 32: (32,)}
+ROWS_TILES = 3040  # from here tile 16 has one adjoint, which stages 32 whatever is asked for (kBwdMinTiles of render.cu)
 TILES = (8, 16, 32)
+
+
+def bwd_batches(tile: int, sizes):
+    """The adjoint's batch depths that differ at this tile size (sizes None: a launch of any size)."""
+    n_tiles = sum(-(-w // tile) * -(-h // tile) for w, h in sizes) if sizes else 0
+    return () if tile == 16 and n_tiles >= ROWS_TILES else BWD_BATCHES[tile]
 
 
 def time_config(g: gs.Gaussians, cams: torch.Tensor, sizes, targets: torch.Tensor, cfg: gs.gs_config,
@@ -76,7 +83,7 @@ def tune(g: gs.Gaussians, cams: torch.Tensor, sizes, targets: torch.Tensor, base
         if ms < best[-1]:
             best = (tile, fb, 0, sched, ms)
     fb = best[1]
-    for bb in BWD_BATCHES[tile]:
+    for bb in bwd_batches(tile, sizes):
         ms = run(tile, fb, bb, sched)
         if ms < best[-1]:
             best = (tile, fb, bb, sched, ms)
