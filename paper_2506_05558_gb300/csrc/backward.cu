@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(32 * kGatherWarps) k_item_partials(
         float4 a[kGatherWin], b[kGatherWin];
         float c[kGatherWin];
     };
-    static_assert(sizeof(Win) % 16 == 0);
+    static_assert(sizeof(Win) % 16 == 0 && kGatherWin % 4 == 0 && kGatherWin <= 4 * 32);
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     Win* win = reinterpret_cast<Win*>(s_raw) + 2 * w;
@@ -103,14 +103,18 @@ __global__ void __launch_bounds__(32 * kGatherWarps) k_item_partials(
             else if (k + 1 < kGatherRuns) fetch(lo[k + 1 < kGatherRuns ? k + 1 : k], hi[k + 1 < kGatherRuns ? k + 1 : k], win[buf ^ 1]);
             else asm volatile("cp.async.commit_group;" ::: "memory");
             asm volatile("cp.async.wait_group 1;" ::: "memory");
+            __syncwarp();
             Win& s = win[buf];
-            if (base < hi[k]) {  // slots that hold no partial become zeros (each lane those that it fetched)
-                const int cnt = (int)min(hi[k] - base, (uint32_t)kGatherWin);
-                for (int j = lane; j < cnt; j += 32)
-                    if (__float_as_uint(s.c[j]) == kNoPartial) {
-                        s.a[j] = s.b[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-                        s.c[j] = 0.f;
-                    }
+            const uint32_t cnt = base < hi[k] ? min(hi[k] - base, (uint32_t)kGatherWin) : 0u;
+            if (4u * lane < cnt) {  // slots that hold no partial become zeros
+                const uint4 c = reinterpret_cast<const uint4*>(s.c)[lane];
+                if (c.x == kNoPartial || c.y == kNoPartial || c.z == kNoPartial || c.w == kNoPartial)
+#pragma unroll
+                    for (int j = 4 * lane; j < 4 * lane + 4; j++)
+                        if (__float_as_uint(s.c[j]) == kNoPartial) {
+                            s.a[j] = s.b[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+                            s.c[j] = 0.f;
+                        }
             }
             __syncwarp();
             if (base < hi[k]) {

@@ -274,7 +274,7 @@ __device__ __forceinline__ int my_long_tiles(const uint32_t* __restrict__ range,
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     unsigned any = 0;
 #pragma unroll 1
-    for (int t0 = 0; t0 < kLongTiles; t0 += kAhead * NT) {
+    for (int t0 = 0; t0 < n_tiles; t0 += kAhead * NT) {
         uint32_t a[kAhead], b[kAhead];
 #pragma unroll
         for (int k = 0; k < kAhead; k++) {
@@ -293,9 +293,9 @@ __device__ __forceinline__ int my_long_tiles(const uint32_t* __restrict__ range,
     if (threadIdx.x == 0) s_n = 0;
     if (!__syncthreads_or(any != 0)) return 0;
     // a tile's rank: the long ones of the words before its own, then of its word
+    const int w0 = threadIdx.x * kPer, w1 = min(w0 + kPer, (n_tiles + 31) / 32);
     int mine = 0;
-#pragma unroll
-    for (int k = 0; k < kPer; k++) mine += __popc(s_mask[threadIdx.x * kPer + k]);
+    for (int q = w0; q < w1; q++) mine += __popc(s_mask[q]);
     int rank = mine;  // inclusive over the warp
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -306,11 +306,11 @@ __device__ __forceinline__ int my_long_tiles(const uint32_t* __restrict__ range,
     __syncthreads();
     rank -= mine;
     for (int q = 0; q < w; q++) rank += s_count[q];
-    for (int k = 0; k < kPer; k++)
-        for (unsigned m = s_mask[threadIdx.x * kPer + k]; m; m &= m - 1, rank++)
+    for (int q = w0; q < w1; q++)
+        for (unsigned m = s_mask[q]; m; m &= m - 1, rank++)
             if (rank % (int)gridDim.x == (int)blockIdx.x) {
                 const int i = atomicAdd(&s_n, 1);
-                if (i < kLongMine) s_mine[i] = 32 * ((int)threadIdx.x * kPer + k) + __ffs(m) - 1;
+                if (i < kLongMine) s_mine[i] = 32 * q + __ffs(m) - 1;
             }
     __syncthreads();
     return min(s_n, kLongMine);
@@ -1022,6 +1022,7 @@ __global__ void __launch_bounds__(32, 16) k_rows_bwd(gs_frame f, gs_config cfg, 
     __shared__ uint16_t s_list[kRowBlocks][kBwdBatch + 1];  // row | block sum << 8
     __shared__ float s_sum[kBwdBatch * kRowBlocks][9];
     __shared__ int s_item;
+    __shared__ int s_tile, s_odd;  // the tile; a sum of it that is not finite
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x, blk = lane >> 2;
     const float inv_log2e = 1.f / kLog2e;
@@ -1035,7 +1036,11 @@ __global__ void __launch_bounds__(32, 16) k_rows_bwd(gs_frame f, gs_config cfg, 
     for (int tile = next_tile(order, counter, n_tiles, true, &s_item); tile >= 0;
          tile = next_tile(order, counter, n_tiles, false, &s_item)) {
         const uint32_t start = range[2 * tile], len = range[2 * tile + 1] - start;
-        if (lane == 0) again[tile] = 0;
+        if (lane == 0) {
+            s_tile = tile;
+            s_odd = 0;
+            again[tile] = 0;
+        }
         if (share > 0.f && len > long_list(count, capacity, share)) continue;  // k_render_bwd's
         const RowInfo ti = row_info(f, tile, aligned);
         const float py = ti.y + 0.5f;
@@ -1264,10 +1269,11 @@ __global__ void __launch_bounds__(32, 16) k_rows_bwd(gs_frame f, gs_config cfg, 
                 part0[em] = make_float4(a[0], a[1], -0.5f * a[4], -a[5]);
                 part1[em] = make_float4(-0.5f * a[2], e.o > 0.f ? a[8] / e.o : 0.f, a[3], a[6]);
                 part2[em] = a[7];
-                if (!(fabsf(a[8]) < INFINITY)) again[tile] = 1;
+                if (!(fabsf(a[8]) < INFINITY)) s_odd = 1;
             }
             __syncwarp();  // rows, lists and sums are rewritten by the next batch
         }
+        if (lane == 0 && s_odd) again[s_tile] = 1;
     }
 }
 
