@@ -613,7 +613,8 @@ int gs_downsample(const float* image, int32_t width, int32_t height, int32_t fac
  * trial cost, accepted) per iteration; *failed (device int32) = 1 if a reduced
  * system was not positive definite (its step is then zero). Everything stays
  * on the device: the call can be captured into a CUDA graph. ws:
- * gs_ba_workspace_size(F, P) bytes. */
+ * gs_ba_workspace_size(F, P) bytes: 12.1 MB at 8 frames x 6144 points, 16.6 GB
+ * at the largest accepted problem (K, V and J of every point are kept). */
 size_t gs_ba_workspace_size(int32_t n_frames, int64_t n_points);
 /* The mini bundle adjustment's camera model: obs [P][F][2] = (fl x/z + cx,
  * fl y/z + cy) of every point in every frame (same layouts as gs_ba_lm). */

@@ -14,7 +14,7 @@ allocator), so several renders may be alive before their backward passes. The
 forward waits once for the host, to grow the (tile, Gaussian) pair buffer when the
 sort reports an overflow (projection, sort and render are launched before it; they
 ran once more for it, on zero-filled buffers, at 1080 us for a forward and backward of
-four 320x180 views of 200k Gaussians, 720 with them gone); the graph-captured training step in raster.py is the
+four 320x180 views of 200k Gaussians, 670 without); the graph-captured training step in raster.py is the
 synchronisation-free path.
 """
 from __future__ import annotations

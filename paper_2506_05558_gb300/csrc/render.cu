@@ -326,7 +326,6 @@ __device__ __forceinline__ int my_long_tiles(const uint32_t* __restrict__ range,
 // each and combine in a fixed order: about a third fewer instructions per hit.
 constexpr int kBwdHits = 8;  // hits per table flush (4 lanes per hit, 8 pixels each)
 
-//
 // LONG: the tiles of a launch of k_rows_bwd that are not for it: those with long lists,
 // beside it, and when it has ended those that it marked (again: a byte per tile).
 template <int TILE, int BB, bool LONG = false>
@@ -743,7 +742,10 @@ __device__ __forceinline__ void composite(FwdPixel& s, float e, float alpha, flo
 // staging (one log2 and two reciprocals instead of two roots and two divisions)
 // 1.30, two hits per loop round 1.21. Four warps per tile leave small launches
 // with too few warps: at 240 tiles 102 against 82 us, at 960 tiles 132 against
-// 133, at 1840 tiles 67 against 78.
+// 133, at 1840 tiles 67 against 78. A tile whose list is many times the others' ends
+// the launch by itself, and an entry of it takes 0.040 us here against 0.029 in
+// k_render_fwd: scenes with deep transparent clusters run at 0.87 to 0.99 of its speed
+// (0.73 with nearly all pairs in a few tiles).
 constexpr int kFwdThreads = 128;
 constexpr int kFwdMinTiles = 1216;
 
@@ -891,9 +893,10 @@ __global__ void __launch_bounds__(kFwdThreads) k_blocks_fwd(gs_frame f, gs_confi
 // pixels - loads, list and loop, the reduction over rows - is paid once per eight
 // blocks.
 //
-// 1M Gaussians, eight 1080p views: 4.43 -> 2.33 ms against k_render_bwd<16, 64>
-// (115 instead of 248 million warp instructions per view; issue 63% busy at 14
-// warps per SM, which registers and the block sums in shared memory allow). Of
+// 1M Gaussians, eight 1080p views: 4.43 -> 2.38 ms against k_render_bwd<16, 64>
+// (248 instead of 535 million warp instructions per view; issue 67% busy at 14
+// warps per SM, which registers and the block sums in shared memory allow; 2.33 ms
+// before non-finite sums were looked for and long lists left out). Of
 // this the exact block test took 3.05 to 2.89 ms, batches of 32 instead of 64
 // with the next rows on their way 2.42, the cheaper staging 2.33. One warp per
 // tile needs many tiles, more of them in several small views, whose full tiles in the
